@@ -48,12 +48,16 @@ __device__ __forceinline__ void basis(const Vec& t, Vec& e1, Vec& e2) {
   e2 = {t.y * e1.z - t.z * e1.y, t.z * e1.x - t.x * e1.z, t.x * e1.y - t.y * e1.x};
 }
 
-// ln |1 + c1.e1 + c2.e2 + t.(c1 x c2)| (see the file comment).
+// c1.e1 + c2.e2 + t.(c1 x c2) = M - 1 (see the file comment), and ln |M|.
+__device__ __forceinline__ float tube_m1(const Vec& c1, const Vec& c2, const Vec& e1, const Vec& e2,
+                                         const Vec& t) {
+  const float cx = c1.y * c2.z - c1.z * c2.y, cy = c1.z * c2.x - c1.x * c2.z, cz = c1.x * c2.y - c1.y * c2.x;
+  return dot3(c1, e1) + dot3(c2, e2) + fmaf(t.x, cx, fmaf(t.y, cy, t.z * cz));
+}
+
 __device__ __forceinline__ float ln_m(const Vec& c1, const Vec& c2, const Vec& e1, const Vec& e2,
                                       const Vec& t) {
-  const float cx = c1.y * c2.z - c1.z * c2.y, cy = c1.z * c2.x - c1.x * c2.z, cz = c1.x * c2.y - c1.y * c2.x;
-  const float m1 = dot3(c1, e1) + dot3(c2, e2) + fmaf(t.x, cx, fmaf(t.y, cy, t.z * cz));
-  return log1p_small(m1);
+  return log1p_small(tube_m1(c1, c2, e1, e2, t));
 }
 
 // Root alpha in [0, 1] of |r + alpha dr| = R on the chord (stable form).

@@ -64,6 +64,20 @@ struct Sample {
   float ne, te, gx, gy, gz;  // n_e, T_e, grad n_e
 };
 
+// Second derivatives of the n_e interpolant at an evaluation point, inside
+// its cell: the Hessian's components in the orthonormal spherical frame
+// there.  The interpolant is linear along each coordinate, so
+//   H_rr = 0, H_tt = f_r / r, H_pp = f_r / r + cot(theta) f_theta / r^2
+// come with the gradient, and the mixed ones need only differences that the
+// gradient forms anyway.  clear: the point lies at least the given offsets
+// away from every face of its cell, so a neighbour within them sees the same
+// polynomial.
+struct Curv {
+  float hrt, hrp, htp, htt, hpp;
+  float inv_r, rho, inv_rho;
+  bool clear;
+};
+
 // atan2 for the grid lookup: the argument is reduced to a = min/max in [0, 1],
 // atan(a) = a P(a^2) with the degree-7 polynomial fitted by csrc/fit_atan.py
 // (max error 3.7e-8 in exact arithmetic, ~2e-7 rad after FP32 rounding), and
@@ -97,10 +111,10 @@ __device__ __forceinline__ float atan2_grid(float y, float x) {
 // only the T_e loads diverge, the evaluation itself stays warp-uniform).
 // sample_cell does the corner loads, the interpolation and the chain rule
 // for cell (i, j, k) at fractions (u, v, w) of the point (x, y, z).
-template <bool kTe>
+template <bool kTe, bool kCurv = false>
 __device__ __forceinline__ Sample sample_cell_t(const GridDev& G, int i, int j, int k, float u, float v, float w,
                                                 float tsel, float inv_dr, float x, float y, float z, float inv_r,
-                                                float rho, float inv_rho, bool want_te) {
+                                                float rho, float inv_rho, bool want_te, Curv* cv = nullptr) {
   Sample s;
   const int cell = (i * (G.n_t - 1) + j) * G.n_p + k;
   float n000, n001, n010, n011, n100, n101, n110, n111;
@@ -127,6 +141,17 @@ __device__ __forceinline__ Sample sample_cell_t(const GridDev& G, int i, int j, 
   s.gx = fmaf(A + B, x, -C * y);
   s.gy = fmaf(A + B, y, C * x);
   s.gz = fmaf(A, z, -D);
+  if (kCurv) {  // (where cv->clear holds, tsel = 1)
+    const float q0 = d01 - d00, q1 = d11 - d10;
+    cv->hrt = inv_r * fmaf(-f_t, inv_r, (e1 - e0) * inv_dr * G.t_inv);
+    cv->hrp = inv_rho * fmaf(-f_p, inv_r, (g1 - g0) * inv_dr * G.p_inv);
+    cv->htp = inv_r * fmaf(fmaf(u, q1 - q0, q0) * G.t_inv, inv_rho * G.p_inv, -C * z);
+    cv->htt = A;
+    cv->hpp = A + B;
+    cv->inv_r = inv_r;
+    cv->rho = rho;
+    cv->inv_rho = inv_rho;
+  }
   s.te = 0.f;
   if (kTe && want_te) {
     float t000, t001, t010, t011, t100, t101, t110, t111;
@@ -169,9 +194,14 @@ __device__ __forceinline__ int radial_cell(const GridDev& G, float r) {
 }
 
 // The field at (x, y, z): trilinear n_e (and T_e when kTe and want_te) and
-// the exact gradient of the n_e interpolant.
-template <bool kTe>
-__device__ __forceinline__ Sample eval_field_t(const GridDev& G, float x, float y, float z, bool want_te) {
+// the exact gradient of the n_e interpolant.  kCurv: also its second
+// derivatives, and whether the point stays clear of its cell's faces by
+// off_r radially and by off along theta and phi (off at most rho / 256: the
+// angles of an offset, and what the second derivatives leave out, are then
+// known well enough; the tests are written so that a NaN fails them).
+template <bool kTe, bool kCurv = false>
+__device__ __forceinline__ Sample eval_field_t(const GridDev& G, float x, float y, float z, bool want_te,
+                                               float off_r = 0.f, float off = 0.f, Curv* cv = nullptr) {
   const float rho2 = fmaf(x, x, y * y);
   const float r2 = fmaf(z, z, rho2);
   const float inv_r = rsqrtf(r2);
@@ -197,7 +227,12 @@ __device__ __forceinline__ Sample eval_field_t(const GridDev& G, float x, float 
   const float pp = ph * G.p_inv;
   const int k = min(max(__float2int_rd(pp), 0), G.n_p - 1);
   const float w = pp - (float)k;
-  return sample_cell_t<kTe>(G, i, j, k, u, v, w, tsel, inv_dr, x, y, z, inv_r, rho, inv_rho, want_te);
+  if (kCurv) {
+    const float ot = off * inv_r, op = off * inv_rho;
+    cv->clear = fabsf(u - 0.5f) <= fmaf(-off_r, inv_dr, 0.5f) && fabsf(v - 0.5f) <= fmaf(-ot, G.t_inv, 0.5f) &&
+                fabsf(w - 0.5f) <= fmaf(-op, G.p_inv, 0.5f) && op <= 1.f / 256.f;
+  }
+  return sample_cell_t<kTe, kCurv>(G, i, j, k, u, v, w, tsel, inv_dr, x, y, z, inv_r, rho, inv_rho, want_te, cv);
 }
 
 __device__ __forceinline__ Sample eval_field(const GridDev& G, float x, float y, float z, bool want_te) {
@@ -540,6 +575,8 @@ struct TraceParams {
   GridDev G;
   float h, h2_6, h_6, h2_12, hrsun;  // step and derived constants, hrsun = h R_sun [cm]
   float eta, eps_fixed;              // eps = eta |dr|, or eps_fixed when > 0
+  int curv;                          // tube area from the field's second derivatives where a step allows it
+  float eps_reach;                   // curv: no neighbour is farther from its ray (else the step retraces them)
   float tau_stop;                    // <= 0: never
   int max_steps;
   int tbc_mode;

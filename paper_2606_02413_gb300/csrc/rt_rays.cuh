@@ -9,8 +9,11 @@
 //       back) and the TAU_STOP / STEP_LIMIT terminations;
 //   (c) completes step i: chord t^i, transverse basis and eps (Eqs. 5, 6, 8),
 //       the new node, and the clip tests against the inner and outer spheres;
-//   (d) retraces step i for every neighbour seeded at r^i +- eps e_j with the
-//       central k^i (Eq. 7) and accumulates ln M^{i+1} (Eqs. 9-11);
+//   (d) accumulates ln M^{i+1} (Eqs. 9-11): from the field's second
+//       derivatives at the central ray's stage points while the neighbours
+//       stay in those points' cells (kCurv, curvature_ln_m), else from a
+//       retrace of step i for every neighbour, seeded at r^i +- eps e_j with
+//       the central k^i (Eq. 7);
 //   (e) on a clipped last step, closes the path at the crossing point.
 // This is the order of the paper's per-step description; the lane-parallel
 // bundle kernel (rt_bundle.cuh) computes the same quantities with the
@@ -22,8 +25,8 @@
 // NB + 1 and took a third of the warp's issue slots.  Here every lane of a
 // warp does useful work in every instruction, and a neighbour needs only the
 // first three RK4 stages (its separation depends on its end position, which
-// does not involve the fourth stage), so a step costs 4 + 3 NB field
-// evaluations instead of 4 (NB + 1).
+// does not involve the fourth stage), so a retraced step costs 4 + 3 NB field
+// evaluations instead of 4 (NB + 1), and one clear of the faces 4.
 //
 // Precision (kMixed) and the offset form of the separations are those of
 // rt_bundle.cuh: d_j = eps e_j + h^2/12 (G_{+j} - G_{-j}) for a +-e_j pair,
@@ -63,13 +66,22 @@ __device__ __forceinline__ Vec rk4_g3(const GridDev& G, float kf, float h, float
 }
 
 // One central RK4 step (see rk4_step) with the stage-1 sample including T_e;
-// stages 1 and 2, and then 3 and 4, are independent of each other.
+// stages 1 and 2, and then 3 and 4, are independent of each other.  kCurv:
+// also the second derivatives at the first three stage points (cv[0..2]),
+// which the neighbours' retrace needs, and those points' clearance.
+struct StagePoints {
+  Curv cv[3];
+  float x2, y2, z2, x3, y3, z3;  // stage points 2 and 3
+};
+template <bool kCurv = false>
 __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float h, float px, float py, float pz,
-                                              float kx, float ky, float kz) {
+                                              float kx, float ky, float kz, float off_r = 0.f, float off = 0.f,
+                                              StagePoints* sp = nullptr) {
   Rk4Out o;
   const float hh = 0.5f * h;
-  const Sample s1 = eval_field_t<true>(G, px, py, pz, true);
-  const Sample s2 = eval_field_t<false>(G, fmaf(hh, kx, px), fmaf(hh, ky, py), fmaf(hh, kz, pz), false);
+  const float x2 = fmaf(hh, kx, px), y2 = fmaf(hh, ky, py), z2 = fmaf(hh, kz, pz);
+  const Sample s1 = eval_field_t<true, kCurv>(G, px, py, pz, true, off_r, off, kCurv ? &sp->cv[0] : nullptr);
+  const Sample s2 = eval_field_t<false, kCurv>(G, x2, y2, z2, false, off_r, off, kCurv ? &sp->cv[1] : nullptr);
   o.ne1 = s1.ne;
   o.te1 = s1.te;
   const float a1x = kf * s1.gx, a1y = kf * s1.gy, a1z = kf * s1.gz;
@@ -81,13 +93,41 @@ __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float 
   // stage 3 at p + h/2 (k + h/2 a1), stage 4 at p + h (k + h/2 a2)
   const float qx = fmaf(hh, a1x, kx), qy = fmaf(hh, a1y, ky), qz = fmaf(hh, a1z, kz);
   const float q3x = fmaf(hh, a2x, kx), q3y = fmaf(hh, a2y, ky), q3z = fmaf(hh, a2z, kz);
-  const Sample s3 = eval_field_t<false>(G, fmaf(hh, qx, px), fmaf(hh, qy, py), fmaf(hh, qz, pz), false);
+  const float x3 = fmaf(hh, qx, px), y3 = fmaf(hh, qy, py), z3 = fmaf(hh, qz, pz);
+  const Sample s3 = eval_field_t<false, kCurv>(G, x3, y3, z3, false, off_r, off, kCurv ? &sp->cv[2] : nullptr);
   const Sample s4 = eval_field_t<false>(G, fmaf(h, q3x, px), fmaf(h, q3y, py), fmaf(h, q3z, pz), false);
   const float a3x = kf * s3.gx, a3y = kf * s3.gy, a3z = kf * s3.gz;
   o.Gx += a3x; o.Gy += a3y; o.Gz += a3z;
   o.Ax = fmaf(2.f, a3x, o.Ax); o.Ay = fmaf(2.f, a3y, o.Ay); o.Az = fmaf(2.f, a3z, o.Az);
   o.Ax = fmaf(kf, s4.gx, o.Ax); o.Ay = fmaf(kf, s4.gy, o.Ay); o.Az = fmaf(kf, s4.gz, o.Az);
+  if (kCurv) {
+    sp->x2 = x2; sp->y2 = y2; sp->z2 = z2;
+    sp->x3 = x3; sp->y3 = y3; sp->z3 = z3;
+  }
   return o;
+}
+
+// How far a step's neighbours reach radially: they sit eps off the path
+// across the chord, so eps sin(angle of the ray to the radius), with 0.01 eps
+// for the turn of the chord and of the radius over the step (the wave vector
+// at the node stands for both) and for the second order eps^2 / 2r.
+__device__ __forceinline__ float radial_reach(float reach, float px, float py, float pz, float kx, float ky, float kz) {
+  const float pk = fmaf(px, kx, fmaf(py, ky, pz * kz));
+  const float pp = fmaf(px, px, fmaf(py, py, pz * pz)), kk = fmaf(kx, kx, fmaf(ky, ky, kz * kz));
+  const float c2 = __fdividef(pk * pk, pp * kk);
+  return reach * (__fsqrt_rn(fmaxf(1.f - c2, 0.f)) + 0.01f);
+}
+
+// Trace of the field's Hessian across the direction t at the point (x, y, z):
+// sum_j e_j.H e_j over a transverse basis = tr H - t.H t.  f: t in the
+// spherical frame there.
+__device__ __forceinline__ float transverse_trace(const Curv& c, float x, float y, float z, const Vec& t, Vec& f) {
+  const float xt = fmaf(x, t.x, y * t.y);
+  f.x = fmaf(z, t.z, xt) * c.inv_r;
+  f.y = fmaf(z * c.inv_rho, xt, -c.rho * t.z) * c.inv_r;
+  f.z = fmaf(x, t.y, -y * t.x) * c.inv_rho;
+  const float cross = fmaf(f.x, fmaf(f.y, c.hrt, f.z * c.hrp), f.y * f.z * c.htp);
+  return fmaf(-2.f, cross, fmaf(c.htt, fmaf(-f.y, f.y, 1.f), c.hpp * fmaf(-f.z, f.z, 1.f)));
 }
 
 // "+" seed offset of neighbour pair j from the node: eps e1, eps e2, and (8
@@ -136,20 +176,54 @@ struct Retrace {
   float eps, lm;
 };
 
+// Chord direction, transverse basis and eps of a step (Eqs. 5, 6, 8).
+__device__ __forceinline__ void chord_frame(Retrace& R, float eta, float eps_fixed, const Vec& dr) {
+  const float d2n = dot3(dr, dr);
+  const float ids = rsqrtf(d2n);
+  R.t = {dr.x * ids, dr.y * ids, dr.z * ids};
+  basis(R.t, R.e1, R.e2);
+  R.eps = (eps_fixed > 0.f) ? eps_fixed : eta * (d2n * ids);
+}
+
+// c1, c2 and ln M from the raw separations D (NB >= 4: D_j = G_{+j} - G_{-j}
+// over the +-pair j; NB == 2: D_j = G_j).
+template <int NB>
+__device__ __forceinline__ void finish_retrace(Retrace& R, const Vec* D, float h2_6, float h2_12, const Vec& G0) {
+  constexpr int NP = (NB >= 4) ? NB / 2 : 2;
+  if (NB == 2) {  // one-sided: d_j = eps e_j + h^2/6 (G_j - G_0)
+    const float sc = h2_6 / R.eps;
+    R.c1 = {sc * (D[0].x - G0.x), sc * (D[0].y - G0.y), sc * (D[0].z - G0.z)};
+    R.c2 = {sc * (D[1].x - G0.x), sc * (D[1].y - G0.y), sc * (D[1].z - G0.z)};
+  } else {        // central difference: d = eps e + h^2/12 (G_+ - G_-)
+    const float sc = h2_12 / R.eps;
+    R.c1 = {sc * D[0].x, sc * D[0].y, sc * D[0].z};
+    R.c2 = {sc * D[1].x, sc * D[1].y, sc * D[1].z};
+  }
+  const float m = tube_m1(R.c1, R.c2, R.e1, R.e2, R.t);
+  R.lm = log1p_small(m);
+  if (NB == 8) {
+    const float s2 = 0.70710678118654752f, sc = h2_12 / R.eps;
+    const Vec g1{s2 * (R.e1.x + R.e2.x), s2 * (R.e1.y + R.e2.y), s2 * (R.e1.z + R.e2.z)};
+    const Vec g2{s2 * (R.e2.x - R.e1.x), s2 * (R.e2.y - R.e1.y), s2 * (R.e2.z - R.e1.z)};
+    const Vec c3{sc * D[2 % NP].x, sc * D[2 % NP].y, sc * D[2 % NP].z};
+    const Vec c4{sc * D[3 % NP].x, sc * D[3 % NP].y, sc * D[3 % NP].z};
+    // M = (M_e + M_g) / 2, taken before the logarithm: the mean of two
+    // logarithms' exponentials would round ln M (~1e-7 a step) at ln 2's ulp
+    const float m2 = tube_m1(c3, c4, g1, g2, R.t);
+    R.lm = (m > -1.f && m2 > -1.f) ? log1p_small(0.5f * (m + m2))
+                                   : __logf(0.5f * (fabsf(1.f + m) + fabsf(1.f + m2)));
+  }
+}
+
 template <int NB>
 __device__ __forceinline__ Retrace retrace_step(const GridDev& G, float kf, float h, float h2_6, float h2_12,
                                                 float eta, float eps_fixed, float px, float py, float pz, float kx,
                                                 float ky, float kz, const Vec& dr, const Vec& G0) {
   Retrace R;
-  const float d2n = dot3(dr, dr);
-  const float ids = rsqrtf(d2n);
-  R.t = {dr.x * ids, dr.y * ids, dr.z * ids};  // chord direction (Eq. 5)
-  basis(R.t, R.e1, R.e2);                      // transverse basis (Eq. 6)
-  R.eps = (eps_fixed > 0.f) ? eps_fixed : eta * (d2n * ids);  // Eq. 8
+  chord_frame(R, eta, eps_fixed, dr);
   const Vec sa{R.eps * R.e1.x, R.eps * R.e1.y, R.eps * R.e1.z}, sb{R.eps * R.e2.x, R.eps * R.e2.y, R.eps * R.e2.z};
-  // raw separations: NB >= 4: D_j = G_{+j} - G_{-j} over the +-pair j
-  // (neighbour q is the "+" (even q) or "-" (odd q) member of pair q / 2);
-  // NB == 2: D_j = G_j.  One retrace per loop trip keeps the code small.
+  // neighbour q is the "+" (even q) or "-" (odd q) member of pair q / 2.
+  // One retrace per loop trip keeps the code small.
   constexpr int NP = (NB >= 4) ? NB / 2 : 2;
   Vec D[NP];
 #pragma unroll
@@ -164,30 +238,110 @@ __device__ __forceinline__ Retrace retrace_step(const GridDev& G, float kf, floa
     for (int m = 0; m < NP; ++m)
       if (m == j) D[m] = {fmaf(sgn, g.x, D[m].x), fmaf(sgn, g.y, D[m].y), fmaf(sgn, g.z, D[m].z)};
   }
-  if (NB == 2) {  // one-sided: d_j = eps e_j + h^2/6 (G_j - G_0)
-    const float sc = h2_6 / R.eps;
-    R.c1 = {sc * (D[0].x - G0.x), sc * (D[0].y - G0.y), sc * (D[0].z - G0.z)};
-    R.c2 = {sc * (D[1].x - G0.x), sc * (D[1].y - G0.y), sc * (D[1].z - G0.z)};
-  } else {        // central difference: d = eps e + h^2/12 (G_+ - G_-)
-    const float sc = h2_12 / R.eps;
-    R.c1 = {sc * D[0].x, sc * D[0].y, sc * D[0].z};
-    R.c2 = {sc * D[1].x, sc * D[1].y, sc * D[1].z};
-  }
-  R.lm = ln_m(R.c1, R.c2, R.e1, R.e2, R.t);
-  if (NB == 8) {
-    const float s2 = 0.70710678118654752f, sc = h2_12 / R.eps;
-    const Vec g1{s2 * (R.e1.x + R.e2.x), s2 * (R.e1.y + R.e2.y), s2 * (R.e1.z + R.e2.z)};
-    const Vec g2{s2 * (R.e2.x - R.e1.x), s2 * (R.e2.y - R.e1.y), s2 * (R.e2.z - R.e1.z)};
-    const Vec c3{sc * D[2 % NP].x, sc * D[2 % NP].y, sc * D[2 % NP].z};
-    const Vec c4{sc * D[3 % NP].x, sc * D[3 % NP].y, sc * D[3 % NP].z};
-    const float lm2 = ln_m(c3, c4, g1, g2, R.t);
-    // M = (M_e + M_g) / 2
-    R.lm = fmaxf(R.lm, lm2) + log1p_small(__expf(-fabsf(R.lm - lm2))) - 0.69314718055994531f;
-  }
+  finish_retrace<NB>(R, D, h2_6, h2_12, G0);
   return R;
 }
 
-template <int NB, bool kMixed>
+// ln M of a step whose neighbours all stay in the cells of the central ray's
+// own stage points.  There a +-pair's separation is, to its third order in
+// eps, the Hessian's: G_+ - G_- = 2 eps kf sum_s H(P_s) e over the three
+// stage points P_s of the central ray, so with C = h^2/6 kf sum_s H(P_s)
+//   ln M = tr_t C - tr_t C^2 / 2 + (tr C^2 - |C t|^2) / 6 + O(C^3),
+// tr_t the trace across t; the last term is the third stage's own shift by
+// h^2/4 a_1.  The same for 4 and for 8 neighbours and for any eps: no
+// neighbour is evaluated.  The second order (formed at the middle stage
+// point) is skipped where |C| <= 1e-5: it is below 1e-10 there; a step with
+// |C| > 1e-3 does not count as small and retraces its neighbours.
+// Why: the neighbours' 12 (24) of a step's 16 (28) field evaluations were
+// three quarters of the kernel's instructions, and it is bound by issue.
+// Twelve second derivatives at points whose cell and fractions the central
+// ray has anyway cost about one evaluation.  One GB300, 4 neighbours, global
+// corona 128^2 x 16 frequencies: 660 ms -> 332 ms; 64^2 x 1 on a 64x32x64
+// corona 14.3 -> 7.9 ms; 8 neighbours, 97x61 x 3: 37.5 -> 11.6 ms.  Paths,
+// optical depths and step counts are bit-identical to the retraced form's;
+// ln S differs by 5.6e-8 (rms) on the global corona.
+__device__ __forceinline__ float curvature_ln_m(const StagePoints& sp, float px, float py, float pz, const Vec& t,
+                                                float h2_6kf, bool& small) {
+  Vec f1, f2, f3;
+  const float q2 = transverse_trace(sp.cv[1], sp.x2, sp.y2, sp.z2, t, f2);
+  const float q = transverse_trace(sp.cv[0], px, py, pz, t, f1) + q2 +
+                  transverse_trace(sp.cv[2], sp.x3, sp.y3, sp.z3, t, f3);
+  const Curv& c = sp.cv[1];
+  const float off = fmaf(c.hrt, c.hrt, fmaf(c.hrp, c.hrp, c.htp * c.htp));
+  const float h2 = fmaf(2.f, off, fmaf(c.htt, c.htt, c.hpp * c.hpp));  // tr H^2
+  const float s2 = 9.f * h2_6kf * h2_6kf;                              // C = 3 h^2/6 kf H there
+  small = s2 * h2 <= 1e-6f;
+  float lm = h2_6kf * q;
+  if (s2 * h2 > 1e-10f) {
+    const float gr = fmaf(c.hrt, f2.y, c.hrp * f2.z), gt = fmaf(c.hrt, f2.x, fmaf(c.htt, f2.y, c.htp * f2.z)),
+                gp = fmaf(c.hrp, f2.x, fmaf(c.htp, f2.y, c.hpp * f2.z));
+    const float g2 = fmaf(gr, gr, fmaf(gt, gt, gp * gp));              // |H t|^2
+    const float th = c.htt + c.hpp - q2;                               // t.H t
+    lm = fmaf(s2, fmaf(1.f / 6.f, h2 - g2, -0.5f * fmaf(th, th, fmaf(-2.f, g2, h2))), lm);
+  }
+  return lm;
+}
+
+// The neighbours of a step that comes too near a face (about one step in
+// ten on a 64x32x64 corona at h = 2e-3, one in twenty on the global one) are
+// retraced; almost every warp has such a lane, so a branch per lane would pay
+// for all of them.  A warp's lanes retrace together the neighbours of the lanes that ask for it
+// (slow): NB lanes per asking lane, one neighbour each, 32 / NB asking lanes
+// at a time.  The arithmetic of each is retrace_step's.  Every lane of the
+// warp calls it; R.t, e1, e2, eps hold the asking lane's frame, and its ln M
+// comes back in R.lm.
+template <int NB>
+struct RetraceSlot {
+  float v[(NB == 8) ? 16 : 13];  // p, k, eps e1, eps e2, kf; then D_1 ... D_{NB/2}
+};
+template <int NB>
+__device__ __forceinline__ void retrace_shared(const GridDev& G, RetraceSlot<NB>* slots, bool slow, float kf, float h,
+                                               float h2_6, float h2_12, float px, float py, float pz, float kx,
+                                               float ky, float kz, Retrace& R) {
+  constexpr int PER = 32 / NB;
+  const int lane = threadIdx.x & 31;
+  const int q = lane % NB, group = lane / NB;
+  unsigned todo = __ballot_sync(kFull, slow);
+  while (todo) {
+    const int rank = __popc(todo & ((1u << lane) - 1u));
+    const bool mine = slow && rank < PER;
+    if (mine) {
+      float* v = slots[rank].v;
+      v[0] = px; v[1] = py; v[2] = pz;
+      v[3] = kx; v[4] = ky; v[5] = kz;
+      v[6] = R.eps * R.e1.x; v[7] = R.eps * R.e1.y; v[8] = R.eps * R.e1.z;
+      v[9] = R.eps * R.e2.x; v[10] = R.eps * R.e2.y; v[11] = R.eps * R.e2.z;
+      v[12] = kf;
+    }
+    __syncwarp();
+    // groups past the last asking lane repeat it (the lookups stay in bounds, nothing is written)
+    const int asking = min(__popc(todo), PER);
+    float* v = slots[min(group, asking - 1)].v;
+    const float sgn = (q & 1) ? -1.f : 1.f;
+    const Vec off = pair_offset(q >> 1, Vec{v[6], v[7], v[8]}, Vec{v[9], v[10], v[11]});
+    const Vec g = rk4_g3(G, v[12], h, fmaf(sgn, off.x, v[0]), fmaf(sgn, off.y, v[1]), fmaf(sgn, off.z, v[2]), v[3],
+                         v[4], v[5]);
+    const Vec d{g.x - __shfl_down_sync(kFull, g.x, 1), g.y - __shfl_down_sync(kFull, g.y, 1),
+                g.z - __shfl_down_sync(kFull, g.z, 1)};
+    __syncwarp();
+    if (group < asking && !(q & 1)) {
+      float* w = v + 3 * (q >> 1);
+      w[0] = d.x; w[1] = d.y; w[2] = d.z;
+    }
+    __syncwarp();
+    if (mine) {
+      Vec D[NB / 2];
+#pragma unroll
+      for (int m = 0; m < NB / 2; ++m)
+        D[m] = {slots[rank].v[3 * m], slots[rank].v[3 * m + 1], slots[rank].v[3 * m + 2]};
+      finish_retrace<NB>(R, D, h2_6, h2_12, Vec{0.f, 0.f, 0.f});
+      slow = false;
+    }
+    todo = __ballot_sync(kFull, slow);
+  }
+}
+
+template <int NB, bool kMixed, bool kCurv>
 __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __grid_constant__ TraceParams P) {
   const int lane = threadIdx.x & 31;
   const float h = P.h;
@@ -202,6 +356,9 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
     int ck_last;  // tape: the ray's last checkpoint slot (-1: none)
   };
   __shared__ Cold cold[kThreads];
+  static_assert(!kCurv || NB >= 4, "the Hessian form stands for +-pairs");
+  constexpr int kSlots = kCurv ? 32 / (NB > 0 ? NB : 1) : 1;
+  __shared__ RetraceSlot<(NB > 0 ? NB : 4)> slots[kThreads / 32][kSlots];
   Cold& C = cold[threadIdx.x];
   C.out = nullptr;
   C.dg = nullptr;
@@ -243,7 +400,9 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
   // uniform registers.
   auto step_once = [&]() {
     // ---------------------------------------------- (a) central RK4 step
-    const Rk4Out o = rk4_central(P.G, kf, h, px, py, pz, kx, ky, kz);
+    StagePoints sp;
+    const float off_r = kCurv ? radial_reach(P.eps_reach, px, py, pz, kx, ky, kz) : 0.f;
+    const Rk4Out o = rk4_central<kCurv>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.eps_reach, &sp);
     const float kap = P.emission ? kappa_vac(o.ne1, o.te1, kap_c, ln_f) : 0.f;
 
     // ---------------------------------------------- (b) segment step-1 -> step
@@ -299,7 +458,17 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
     else if (!isfinite(rr2 + kn.x + kn.y + kn.z)) term = kNan;
 
     // ---------------------------------------------- (d) neighbour retrace of step `step`
-    if (NB > 0) {
+    if constexpr (kCurv) {
+      Retrace R;
+      chord_frame(R, P.eta, P.eps_fixed, dr);
+      bool small;
+      R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, small);
+      const bool counts = stop == 0 && term != kNan;
+      const bool fast = sp.cv[0].clear && sp.cv[1].clear && sp.cv[2].clear && small && R.eps <= P.eps_reach;
+      retrace_shared<NB>(P.G, slots[threadIdx.x >> 5], active && counts && !fast, kf, h, P.h2_6,
+                                       P.h2_12, px, py, pz, kx, ky, kz, R);
+      if (counts) acc_add<kMixed>(lns_hi, lns_lo, R.lm);
+    } else if (NB > 0) {
       const Retrace R = retrace_step<NB>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky, kz,
                                          dr, Vec{o.Gx, o.Gy, o.Gz});
       if (stop == 0 && term != kNan) acc_add<kMixed>(lns_hi, lns_lo, R.lm);
@@ -412,7 +581,7 @@ struct PathNode {
 // them (the same step code in the same order), recording every node.
 // The first `cap` nodes of ray i go to path[i * cap ...], its node count to
 // count[i], and its T_b and diagnostics to tb[i] and diag[i].
-template <int NB, bool kMixed>
+template <int NB, bool kMixed, bool kCurv>
 __global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceParams P, const int* __restrict__ pix,
                                                   int n, int cap, PathNode* __restrict__ path, int* __restrict__ count,
                                                   float* __restrict__ tb, RayDiag* __restrict__ diag) {
@@ -442,7 +611,9 @@ __global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceP
     float rlx = 0.f, rly = 0.f, rlz = 0.f, klx = 0.f, kly = 0.f, klz = 0.f;
     float kap_prev = 0.f, te_prev = 0.f, dls = 0.f;
     while (true) {
-      const Rk4Out o = rk4_central(P.G, kf, h, px, py, pz, kx, ky, kz);
+      StagePoints sp;
+      const float off_r = kCurv ? radial_reach(P.eps_reach, px, py, pz, kx, ky, kz) : 0.f;
+      const Rk4Out o = rk4_central<kCurv>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.eps_reach, &sp);
       const float kap = P.emission ? kappa_vac(o.ne1, o.te1, kap_c, ln_f) : 0.f;
       if (step >= 1) {
         const float dt = 0.5f * (kap_prev + kap) * P.hrsun;
@@ -466,8 +637,17 @@ __global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceP
       else if (!isfinite(rr2 + kn.x + kn.y + kn.z)) term = kNan;
       dls = 0.f;
       if (NB > 0 && term != kNan) {
-        const Retrace R = retrace_step<(NB > 0 ? NB : 4)>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py,
-                                                          pz, kx, ky, kz, dr, Vec{o.Gx, o.Gy, o.Gz});
+        Retrace R;
+        bool fast = false;
+        if (kCurv) {
+          chord_frame(R, P.eta, P.eps_fixed, dr);
+          bool small;
+          R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, small);
+          fast = sp.cv[0].clear && sp.cv[1].clear && sp.cv[2].clear && small && R.eps <= P.eps_reach;
+        }
+        if (!fast)
+          R = retrace_step<(NB > 0 ? NB : 4)>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky,
+                                              kz, dr, Vec{o.Gx, o.Gy, o.Gz});
         acc_add<kMixed>(lns_hi, lns_lo, R.lm);
         dls = R.lm * rsqrtf(dot3(dr, dr));
       }
