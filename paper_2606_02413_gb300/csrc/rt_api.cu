@@ -235,9 +235,9 @@ __global__ void __launch_bounds__(kBeamThreads) beam_pass(const float* __restric
   // offsets that reach a pixel of the image from some pixel of the tile
   const int n = kCol ? B.ny : B.nx, a0 = kCol ? y0 : x0, ta = kCol ? TY : TX;
   const int lo_d = max(-hw, -(a0 + ta - 1)), hi_d = min(hw, n - 1 - a0);
-  float hi[kBeamOut], lo[kBeamOut];
+  F2 hi2[kBeamOut / 2], lo2[kBeamOut / 2];
 #pragma unroll
-  for (int i = 0; i < kBeamOut; ++i) hi[i] = lo[i] = 0.f;
+  for (int i = 0; i < kBeamOut / 2; ++i) hi2[i] = lo2[i] = f2(0.f);
   for (int d0 = lo_d; d0 <= hi_d; d0 += kBeamTaps) {
     const int nt = min(kBeamTaps, hi_d - d0 + 1);
     __syncthreads();
@@ -254,16 +254,26 @@ __global__ void __launch_bounds__(kBeamThreads) beam_pass(const float* __restric
     __syncthreads();
     for (int t = 0; t < nt; ++t) {
       const float w = wgt[t];
+      const F2 w2 = f2(w), wn2 = f2(-w);
 #pragma unroll
-      for (int i = 0; i < kBeamOut; ++i) {
-        const float v = kCol ? tile[row + i * (kBeamThreads / 32) + t][lane] : tile[row][lane + 32 * i + t];
-        const float p = w * v, e = fmaf(w, v, -p);
-        float s, r;
-        two_sum(hi[i], p, s, r);
-        hi[i] = s;
-        lo[i] += r + e;
+      for (int i = 0; i < kBeamOut / 2; ++i) {
+        auto at = [&](int k) {
+          return kCol ? tile[row + k * (kBeamThreads / 32) + t][lane] : tile[row][lane + 32 * k + t];
+        };
+        // p = w v, e = w v - p; s = hi + p, r its rounding (TwoSum); np = -p
+        const F2 v = f2(at(2 * i), at(2 * i + 1)), np = mul2(wn2, v), e = fma2(w2, v, np);
+        const F2 s = sub2(hi2[i], np), b = sub2(s, hi2[i]);
+        const F2 r = sub2(sub2(hi2[i], sub2(s, b)), add2(b, np));
+        hi2[i] = s;
+        lo2[i] = add2(lo2[i], add2(r, e));
       }
     }
+  }
+  float hi[kBeamOut], lo[kBeamOut];
+#pragma unroll
+  for (int i = 0; i < kBeamOut / 2; ++i) {
+    unpack(hi2[i], hi[2 * i], hi[2 * i + 1]);
+    unpack(lo2[i], lo[2 * i], lo[2 * i + 1]);
   }
 #pragma unroll
   for (int i = 0; i < kBeamOut; ++i) {
