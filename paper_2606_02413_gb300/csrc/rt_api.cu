@@ -371,18 +371,6 @@ int blocks_per_sm() {
   return cached;
 }
 
-template <int NB, bool M>
-int adj_blocks_per_sm() {
-  static int cached = -1;
-  if (cached < 0) {
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, adjoint_rays<NB, M>, kThreads, 0) != cudaSuccess || b < 1)
-      b = 1;
-    cached = b;
-  }
-  return cached;
-}
-
 template <int NB, bool M, bool C>
 int ray_blocks_per_sm() {
   static int cached = -1;
@@ -1195,7 +1183,7 @@ cudaError_t launch_adjoint(rt_ctx* ctx, const rt_grid* g, const TraceParams& P, 
   std::memset(&A, 0, sizeof A);
   A.G = g->dev;
   A.h = P.h; A.h2_6 = P.h2_6; A.h_6 = P.h_6; A.h2_12 = P.h2_12; A.hrsun = P.hrsun;
-  A.eta = P.eta; A.eps_fixed = P.eps_fixed; A.tbc_K = P.tbc_K; A.tbc_mode = P.tbc_mode; A.emission = P.emission;
+  A.eta = P.eta; A.eps_fixed = P.eps_fixed; A.eps_reach = P.eps_reach; A.curv = P.curv; A.tbc_K = P.tbc_K; A.tbc_mode = P.tbc_mode; A.emission = P.emission;
   A.view = P.view;
   A.nf = P.nf;
   for (int i = 0; i < P.nf; ++i) A.freq[i] = P.freq[i];
@@ -1210,15 +1198,13 @@ cudaError_t launch_adjoint(rt_ctx* ctx, const rt_grid* g, const TraceParams& P, 
   A.counter = ctx->d_counter;
   A.total = P.total;
   A.mismatch = mismatch;
-  const int per_sm = (nb == 0) ? (mixed ? adj_blocks_per_sm<0, true>() : adj_blocks_per_sm<0, false>())
-                               : (mixed ? adj_blocks_per_sm<4, true>() : adj_blocks_per_sm<4, false>());
-  const int grid_blocks = ctx->sm_count * per_sm;
+  const int blocks = ctx->sm_count;  // one block an SM
   if (nb == 0) {
-    if (mixed) adjoint_rays<0, true><<<grid_blocks, kThreads, 0, s>>>(A);
-    else adjoint_rays<0, false><<<grid_blocks, kThreads, 0, s>>>(A);
+    if (mixed) adjoint_rays<0, true><<<blocks, kAdjThreads, 0, s>>>(A);
+    else adjoint_rays<0, false><<<blocks, kAdjThreads, 0, s>>>(A);
   } else {
-    if (mixed) adjoint_rays<4, true><<<grid_blocks, kThreads, 0, s>>>(A);
-    else adjoint_rays<4, false><<<grid_blocks, kThreads, 0, s>>>(A);
+    if (mixed) adjoint_rays<4, true><<<blocks, kAdjThreads, 0, s>>>(A);
+    else adjoint_rays<4, false><<<blocks, kAdjThreads, 0, s>>>(A);
   }
   return cudaGetLastError();
 }

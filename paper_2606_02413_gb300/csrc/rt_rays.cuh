@@ -71,7 +71,8 @@ __device__ __forceinline__ Vec rk4_g3(const GridDev& G, float kf, float h, float
 // which the neighbours' retrace needs, and those points' clearance.
 struct StagePoints {
   Curv cv[3];
-  float x2, y2, z2, x3, y3, z3;  // stage points 2 and 3
+  float x2, y2, z2, x3, y3, z3, x4, y4, z4;  // stage points 2 to 4
+  __device__ __forceinline__ bool clear() const { return cv[0].clear && cv[1].clear && cv[2].clear; }
 };
 template <bool kCurv = false>
 __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float h, float px, float py, float pz,
@@ -95,14 +96,16 @@ __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float 
   const float q3x = fmaf(hh, a2x, kx), q3y = fmaf(hh, a2y, ky), q3z = fmaf(hh, a2z, kz);
   const float x3 = fmaf(hh, qx, px), y3 = fmaf(hh, qy, py), z3 = fmaf(hh, qz, pz);
   const Sample s3 = eval_field_t<false, kCurv>(G, x3, y3, z3, false, off_r, off, kCurv ? &sp->cv[2] : nullptr);
-  const Sample s4 = eval_field_t<false>(G, fmaf(h, q3x, px), fmaf(h, q3y, py), fmaf(h, q3z, pz), false);
+  const float x4 = fmaf(h, q3x, px), y4 = fmaf(h, q3y, py), z4 = fmaf(h, q3z, pz);
+  const Sample s4 = eval_field_t<false>(G, x4, y4, z4, false);
   const float a3x = kf * s3.gx, a3y = kf * s3.gy, a3z = kf * s3.gz;
   o.Gx += a3x; o.Gy += a3y; o.Gz += a3z;
   o.Ax = fmaf(2.f, a3x, o.Ax); o.Ay = fmaf(2.f, a3y, o.Ay); o.Az = fmaf(2.f, a3z, o.Az);
   o.Ax = fmaf(kf, s4.gx, o.Ax); o.Ay = fmaf(kf, s4.gy, o.Ay); o.Az = fmaf(kf, s4.gz, o.Az);
-  if (kCurv) {
+  if (sp) {
     sp->x2 = x2; sp->y2 = y2; sp->z2 = z2;
     sp->x3 = x3; sp->y3 = y3; sp->z3 = z3;
+    sp->x4 = x4; sp->y4 = y4; sp->z4 = z4;
   }
   return o;
 }
@@ -250,8 +253,8 @@ __device__ __forceinline__ Retrace retrace_step(const GridDev& G, float kf, floa
 // tr_t the trace across t; the last term is the third stage's own shift by
 // h^2/4 a_1.  The same for 4 and for 8 neighbours and for any eps: no
 // neighbour is evaluated.  The second order (formed at the middle stage
-// point) is skipped where |C| <= 1e-5: it is below 1e-10 there; a step with
-// |C| > 1e-3 does not count as small and retraces its neighbours.
+// point) is skipped where |C| <= 1e-5: it is below 1e-10 there; c2 = |C|^2: a
+// step with |C| > 1e-3 retraces its neighbours.
 // Why: the neighbours' 12 (24) of a step's 16 (28) field evaluations were
 // three quarters of the kernel's instructions, and it is bound by issue.
 // Twelve second derivatives at points whose cell and fractions the central
@@ -261,7 +264,7 @@ __device__ __forceinline__ Retrace retrace_step(const GridDev& G, float kf, floa
 // optical depths and step counts are bit-identical to the retraced form's;
 // ln S differs by 5.6e-8 (rms) on the global corona.
 __device__ __forceinline__ float curvature_ln_m(const StagePoints& sp, float px, float py, float pz, const Vec& t,
-                                                float h2_6kf, bool& small) {
+                                                float h2_6kf, float& c2) {
   Vec f1, f2, f3;
   const float q2 = transverse_trace(sp.cv[1], sp.x2, sp.y2, sp.z2, t, f2);
   const float q = transverse_trace(sp.cv[0], px, py, pz, t, f1) + q2 +
@@ -270,9 +273,9 @@ __device__ __forceinline__ float curvature_ln_m(const StagePoints& sp, float px,
   const float off = fmaf(c.hrt, c.hrt, fmaf(c.hrp, c.hrp, c.htp * c.htp));
   const float h2 = fmaf(2.f, off, fmaf(c.htt, c.htt, c.hpp * c.hpp));  // tr H^2
   const float s2 = 9.f * h2_6kf * h2_6kf;                              // C = 3 h^2/6 kf H there
-  small = s2 * h2 <= 1e-6f;
+  c2 = s2 * h2;
   float lm = h2_6kf * q;
-  if (s2 * h2 > 1e-10f) {
+  if (c2 > 1e-10f) {
     const float gr = fmaf(c.hrt, f2.y, c.hrp * f2.z), gt = fmaf(c.hrt, f2.x, fmaf(c.htt, f2.y, c.htp * f2.z)),
                 gp = fmaf(c.hrp, f2.x, fmaf(c.htp, f2.y, c.hpp * f2.z));
     const float g2 = fmaf(gr, gr, fmaf(gt, gt, gp * gp));              // |H t|^2
@@ -337,6 +340,7 @@ __device__ __forceinline__ void retrace_shared(const GridDev& G, RetraceSlot<NB>
       finish_retrace<NB>(R, D, h2_6, h2_12, Vec{0.f, 0.f, 0.f});
       slow = false;
     }
+    __syncwarp();  // the slots are read: the next lanes may fill them
     todo = __ballot_sync(kFull, slow);
   }
 }
@@ -461,10 +465,10 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
     if constexpr (kCurv) {
       Retrace R;
       chord_frame(R, P.eta, P.eps_fixed, dr);
-      bool small;
-      R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, small);
+      float c2;
+      R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
       const bool counts = stop == 0 && term != kNan;
-      const bool fast = sp.cv[0].clear && sp.cv[1].clear && sp.cv[2].clear && small && R.eps <= P.eps_reach;
+      const bool fast = sp.clear() && c2 <= 1e-6f && R.eps <= P.eps_reach;
       retrace_shared<NB>(P.G, slots[threadIdx.x >> 5], active && counts && !fast, kf, h, P.h2_6,
                                        P.h2_12, px, py, pz, kx, ky, kz, R);
       if (counts) acc_add<kMixed>(lns_hi, lns_lo, R.lm);
@@ -641,9 +645,9 @@ __global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceP
         bool fast = false;
         if (kCurv) {
           chord_frame(R, P.eta, P.eps_fixed, dr);
-          bool small;
-          R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, small);
-          fast = sp.cv[0].clear && sp.cv[1].clear && sp.cv[2].clear && small && R.eps <= P.eps_reach;
+          float c2;
+          R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
+          fast = sp.clear() && c2 <= 1e-6f && R.eps <= P.eps_reach;
         }
         if (!fast)
           R = retrace_step<(NB > 0 ? NB : 4)>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky,
