@@ -437,6 +437,7 @@ struct AdjParams {
   float* dte;
   unsigned int* counter;
   unsigned int total;
+  int lanes;                     // rays of a warp (32 unless the launch has fewer rays than thread slots)
   unsigned long long* mismatch;  // rays whose step count does not match their checkpoint allocation
 };
 
@@ -513,7 +514,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_rays(const __grid_cons
 
   // per-ray state of the reverse sweep
   unsigned int item = 0;
-  bool active = false, exhausted = false;
+  bool active = false, exhausted = lane >= P.lanes;
   int N = 0, status = 0, seg = 0;
   int slot = -1;  // tape: the pool slot of segment seg's checkpoint
   bool clipped = false;

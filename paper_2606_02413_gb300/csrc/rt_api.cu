@@ -383,12 +383,36 @@ int ray_blocks_per_sm() {
   return cached;
 }
 
+// How a launch of `total` bundles spreads over the GPU when they are fewer than
+// its slots: as many warps as fill every scheduler (4 an SM) evenly, each with
+// only its share of the bundles, instead of full warps on the few SMs whose
+// blocks take their tickets first.  A warp alone on its scheduler takes a step
+// about as fast with 7 bundles as with 32, and two on one scheduler share it.
+// Measured with full warps and with this (one GB300): 64^2 x 1 map 7.9 ->
+// 6.0 ms, 97x61 x 3 with 8 neighbours 11.6 -> 8.2 ms, 96^2 x 2 of a 30 R_sun
+// corona with its load 83 -> 63 ms, a fit step on 40^2 x 2 55 -> 39 ms.
+struct Spread {
+  int warps;  // warps of the launch
+  int lanes;  // bundles of a warp at a time
+};
+Spread spread(unsigned total, int per_warp, int sm_count, int warps_per_sm) {
+  const long schedulers = 4L * sm_count, cap = (long)sm_count * warps_per_sm;
+  const long rounds = ((long)total + schedulers * per_warp - 1) / (schedulers * per_warp);  // warps of a scheduler
+  if (rounds * schedulers >= cap) return {(int)cap, per_warp};
+  const long warps = std::max(1L, rounds) * schedulers;
+  const int lanes = (int)std::max(1L, ((long)total + warps - 1) / warps);
+  return {(int)std::max(1L, ((long)total + lanes - 1) / lanes), lanes};
+}
+
 // tube mode: the lane-parallel bundle kernel (persistent neighbours)
 template <int NB, bool M>
 cudaError_t launch_tube(const TraceParams& P, int sm_count, cudaStream_t s) {
   const int fit = blocks_per_sm<NB, M, true>();
   const int per_sm = (P.blocks_per_sm > 0) ? std::min(P.blocks_per_sm, fit) : fit;
-  trace_bundles<NB, M, true><<<sm_count * per_sm, kThreads, 0, s>>>(P);
+  const Spread sp = spread(P.total, 32 / (NB + 1), sm_count, per_sm * (kThreads / 32));
+  TraceParams Q = P;
+  Q.lanes = sp.lanes;
+  trace_bundles<NB, M, true><<<(sp.warps * 32 + kThreads - 1) / kThreads, kThreads, 0, s>>>(Q);
   return cudaGetLastError();
 }
 
@@ -401,7 +425,10 @@ cudaError_t launch_rays(const TraceParams& P, int sm_count, cudaStream_t s) {
   }
   const int fit = ray_blocks_per_sm<NB, M, C>();
   const int per_sm = (P.blocks_per_sm > 0) ? std::min(P.blocks_per_sm, fit) : fit;
-  trace_rays<NB, M, C><<<sm_count * per_sm, kThreads, 0, s>>>(P);
+  const Spread sp = spread(P.total, 32, sm_count, per_sm * (kThreads / 32));
+  TraceParams Q = P;
+  Q.lanes = sp.lanes;
+  trace_rays<NB, M, C><<<(sp.warps * 32 + kThreads - 1) / kThreads, kThreads, 0, s>>>(Q);
   return cudaGetLastError();
 }
 
@@ -1198,13 +1225,17 @@ cudaError_t launch_adjoint(rt_ctx* ctx, const rt_grid* g, const TraceParams& P, 
   A.counter = ctx->d_counter;
   A.total = P.total;
   A.mismatch = mismatch;
-  const int blocks = ctx->sm_count;  // one block an SM
+  // one block of up to kAdjThreads per SM, with the warps that the rays need
+  const Spread sp = spread(P.total, 32, ctx->sm_count, kAdjThreads / 32);
+  A.lanes = sp.lanes;
+  const int warps = (sp.warps + ctx->sm_count - 1) / ctx->sm_count;  // of a block
+  const int blocks = (sp.warps + warps - 1) / warps;
   if (nb == 0) {
-    if (mixed) adjoint_rays<0, true><<<blocks, kAdjThreads, 0, s>>>(A);
-    else adjoint_rays<0, false><<<blocks, kAdjThreads, 0, s>>>(A);
+    if (mixed) adjoint_rays<0, true><<<blocks, warps * 32, 0, s>>>(A);
+    else adjoint_rays<0, false><<<blocks, warps * 32, 0, s>>>(A);
   } else {
-    if (mixed) adjoint_rays<4, true><<<blocks, kAdjThreads, 0, s>>>(A);
-    else adjoint_rays<4, false><<<blocks, kAdjThreads, 0, s>>>(A);
+    if (mixed) adjoint_rays<4, true><<<blocks, warps * 32, 0, s>>>(A);
+    else adjoint_rays<4, false><<<blocks, warps * 32, 0, s>>>(A);
   }
   return cudaGetLastError();
 }

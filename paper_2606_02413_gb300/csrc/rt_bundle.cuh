@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
   bool has_seed = false;  // neighbour lanes: a retrace is pending
   int phase = 0;          // central: 0 needs work, 1 stepping, 2 final (clipped) segment
   bool emitted = false;   // central: its neighbours retrace a step this iteration
-  bool exhausted = !central;
+  bool exhausted = !central || lane / L >= P.lanes;
   bool fresh = false;     // central (tube mode): a ray started in this iteration
   // tube neighbours (mixed form): rounding carried by the offset accumulation
   float lpx = 0.f, lpy = 0.f, lpz = 0.f, lkx = 0.f, lky = 0.f, lkz = 0.f;

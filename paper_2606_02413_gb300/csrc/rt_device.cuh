@@ -630,6 +630,7 @@ struct TraceParams {
   unsigned int* counter;            // work queue ticket (zeroed before launch)
   unsigned long long* stats;        // [0] ray steps, [1] rays
   unsigned int total;               // tickets
+  int lanes;                        // bundles of a warp (as many as fit unless the launch has fewer bundles than slots)
   // optional checkpoints (image mode): ray t owns ckpt[ck_off[t] .. ck_off[t+1]);
   // or, when ck_prev is set (a tape), each checkpoint takes the next pool slot
   // (pool_counter, at most pool_cap), ck_prev links it to the ray's previous

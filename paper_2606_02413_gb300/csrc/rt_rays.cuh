@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
   C.item = 0;
   C.ck_last = -1;
   int step = 0;
-  bool active = false, exhausted = false;
+  bool active = false, exhausted = lane >= P.lanes;
   float px = 0.f, py = 0.f, pz = 0.f, kx = 0.f, ky = 0.f, kz = 0.f;
   float rlx = 0.f, rly = 0.f, rlz = 0.f, klx = 0.f, kly = 0.f, klz = 0.f;  // compensation (kMixed)
   float kf = 0.f, kap_c = 0.f, ln_f = 0.f;
