@@ -94,8 +94,8 @@ __device__ __forceinline__ Vec value_adjoint(const GridDev& G, float x, float y,
   const int cell = (c.i * (G.n_t - 1) + c.j) * G.n_p + c.k;
   const float4 n0 = __ldg(G.ne + 2 * cell), n1 = __ldg(G.ne + 2 * cell + 1);
   const float4 t0 = __ldg(G.te + 2 * cell), t1 = __ldg(G.te + 2 * cell + 1);
-  const float nv[8] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w};
-  const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+  const float nv[8] = {n0.x, n0.z, n1.x, n1.z, n0.y, n0.w, n1.y, n1.w};  // [a][b][c]
+  const float tv[8] = {t0.x, t0.z, t1.x, t1.z, t0.y, t0.w, t1.y, t1.w};
   const float wu[2] = {1.f - c.u, c.u}, wv[2] = {1.f - c.v, c.v}, ww[2] = {1.f - c.w, c.w};
   const float sg[2] = {-1.f, 1.f};
   float fu = 0.f, fv = 0.f, fw = 0.f, tu = 0.f, tvv = 0.f, tw = 0.f;
@@ -194,7 +194,7 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
 
   // partials of the interpolant in (u, v, w), then in (r, theta, phi)
   float n000, n001, n010, n011, n100, n101, n110, n111;
-  ldg8(G.ne + 2 * cell, n000, n001, n010, n011, n100, n101, n110, n111);
+  ldg8(G.ne + 2 * cell, n000, n100, n001, n101, n010, n110, n011, n111);
   const float d00 = n001 - n000, d01 = n011 - n010, d10 = n101 - n100, d11 = n111 - n110;
   const float a00 = fmaf(w, d00, n000), a01 = fmaf(w, d01, n010), a10 = fmaf(w, d10, n100), a11 = fmaf(w, d11, n110);
   const float e0 = a01 - a00, e1 = a11 - a10;
@@ -279,7 +279,7 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
   if (value) {
     wn = lam_ne;
     float m000, m001, m010, m011, m100, m101, m110, m111;
-    ldg8(G.te + 2 * cell, m000, m001, m010, m011, m100, m101, m110, m111);
+    ldg8(G.te + 2 * cell, m000, m100, m001, m101, m010, m110, m011, m111);
     const float b00 = fmaf(w, m001 - m000, m000), b01 = fmaf(w, m011 - m010, m010);
     const float b10 = fmaf(w, m101 - m100, m100), b11 = fmaf(w, m111 - m110, m110);
     const float t_r = (fmaf(v, b11 - b10, b10) - fmaf(v, b01 - b00, b00)) * inv_dr;
@@ -616,8 +616,9 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_rays(const __grid_cons
         rc.p4[0] = sp.x4; rc.p4[1] = sp.y4; rc.p4[2] = sp.z4;
         rc.kap = kap; rc.te = o.te1; rc.ne = o.ne1;
       }
-      Vec dr, rn, kn;
-      complete_step<kMixed>(h, P.h2_6, P.h_6, o, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, dr, rn, kn);
+      const Vec dr = chord(h, P.h2_6, o, kx, ky, kz, klx, kly, klz);
+      Vec rn, kn;
+      complete_step<kMixed>(P.h_6, o, dr, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, rn, kn);
       if (live) { rc.dr[0] = dr.x; rc.dr[1] = dr.y; rc.dr[2] = dr.z; }
       if constexpr (NB > 0) {
         Retrace T;

@@ -130,8 +130,8 @@ __global__ void pack_cells(const T* __restrict__ ne, const T* __restrict__ te, f
       for (int b = 0; b < 2; ++b)
         for (int cc = 0; cc < 2; ++cc) {
           const long id = ((long)(i + a) * n_t + (j + b)) * n_p + (cc ? k1 : k);
-          vn[a * 4 + b * 2 + cc] = (float)ne[id];
-          vt[a * 4 + b * 2 + cc] = (float)te[id];
+          vn[b * 4 + cc * 2 + a] = (float)ne[id];
+          vt[b * 4 + cc * 2 + a] = (float)te[id];
         }
     cne[2 * c] = make_float4(vn[0], vn[1], vn[2], vn[3]);
     cne[2 * c + 1] = make_float4(vn[4], vn[5], vn[6], vn[7]);

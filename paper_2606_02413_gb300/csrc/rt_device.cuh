@@ -18,8 +18,10 @@ constexpr int kMinBlocksTube = 6;          // tube bundles: the offset evaluatio
 
 // ------------------------------------------------------------------ grid
 // Cells are corner-packed: cell (i, j, k) stores the 8 node values of its
-// corners as two float4, corner index a*4 + b*2 + c for the (r, theta, phi)
-// offsets (a, b, c), so one evaluation is one 32-byte load of one sector.
+// corners as two float4, corner index b*4 + c*2 + a for the (r, theta, phi)
+// offsets (a, b, c), so one evaluation is one 32-byte load of one sector, and
+// each register pair of the load holds the two radial neighbours, which the
+// interpolation along phi and theta treats alike (F2).
 // Cell k = n_phi - 1 wraps to node 0 (phi is periodic).
 //
 // The radial axis (any monotone spacing) is resolved by bins no wider than
@@ -92,6 +94,18 @@ __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
 }
 __device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, f2(-1.f), a); }
 
+// One cell's corners as r-pairs: q[2 b + c] = (value at (0, b, c), at (1, b, c)).
+struct Corners {
+  F2 q[4];
+};
+__device__ __forceinline__ Corners ldg_corners(const float4* p) {
+  Corners c;
+  asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];"
+      : "=l"(c.q[0].v), "=l"(c.q[1].v), "=l"(c.q[2].v), "=l"(c.q[3].v)
+      : "l"(p));
+  return c;
+}
+
 struct Sample {
   float ne, te, gx, gy, gz;  // n_e, T_e, grad n_e
 };
@@ -149,17 +163,18 @@ __device__ __forceinline__ Sample sample_cell_t(const GridDev& G, int i, int j, 
                                                 float rho, float inv_rho, bool want_te, Curv* cv = nullptr) {
   Sample s;
   const int cell = (i * (G.n_t - 1) + j) * G.n_p + k;
-  float n000, n001, n010, n011, n100, n101, n110, n111;
-  ldg8(G.ne + 2 * cell, n000, n001, n010, n011, n100, n101, n110, n111);
-  const float d00 = n001 - n000, d01 = n011 - n010, d10 = n101 - n100, d11 = n111 - n110;
-  const float a00 = fmaf(w, d00, n000), a01 = fmaf(w, d01, n010);
-  const float a10 = fmaf(w, d10, n100), a11 = fmaf(w, d11, n110);
-  const float e0 = a01 - a00, e1 = a11 - a10;
-  const float b0 = fmaf(v, e0, a00), b1 = fmaf(v, e1, a10);
+  const Corners N = ldg_corners(G.ne + 2 * cell);
+  const F2 w2 = f2(w), v2 = f2(v);
+  const F2 D0 = sub2(N.q[1], N.q[0]), D1 = sub2(N.q[3], N.q[2]);          // differences along phi
+  const F2 A0 = fma2(w2, D0, N.q[0]), E = sub2(fma2(w2, D1, N.q[2]), A0);  // values at w, along theta
+  float e0, e1, b0, b1, g0, g1;
+  unpack(E, e0, e1);
+  unpack(fma2(v2, E, A0), b0, b1);
+  const F2 Q = sub2(D1, D0);
+  unpack(fma2(v2, Q, D0), g0, g1);
   const float fu = b1 - b0;
   s.ne = fmaf(u, fu, b0);
   const float fv = fmaf(u, e1 - e0, e0);
-  const float g0 = fmaf(v, d01 - d00, d00), g1 = fmaf(v, d11 - d10, d10);
   const float fw = fmaf(u, g1 - g0, g0);
 
   const float f_r = fu * inv_dr;
@@ -174,7 +189,8 @@ __device__ __forceinline__ Sample sample_cell_t(const GridDev& G, int i, int j, 
   s.gy = fmaf(A + B, y, C * x);
   s.gz = fmaf(A, z, -D);
   if (kCurv) {  // (where cv->clear holds, tsel = 1)
-    const float q0 = d01 - d00, q1 = d11 - d10;
+    float q0, q1;
+    unpack(Q, q0, q1);
     cv->hrt = inv_r * fmaf(-f_t, inv_r, (e1 - e0) * inv_dr * G.t_inv);
     cv->hrp = inv_rho * fmaf(-f_p, inv_r, (g1 - g0) * inv_dr * G.p_inv);
     cv->htp = inv_r * fmaf(fmaf(u, q1 - q0, q0) * G.t_inv, inv_rho * G.p_inv, -C * z);
@@ -186,11 +202,10 @@ __device__ __forceinline__ Sample sample_cell_t(const GridDev& G, int i, int j, 
   }
   s.te = 0.f;
   if (kTe && want_te) {
-    float t000, t001, t010, t011, t100, t101, t110, t111;
-    ldg8(G.te + 2 * cell, t000, t001, t010, t011, t100, t101, t110, t111);
-    const float p00 = fmaf(w, t001 - t000, t000), p01 = fmaf(w, t011 - t010, t010);
-    const float p10 = fmaf(w, t101 - t100, t100), p11 = fmaf(w, t111 - t110, t110);
-    const float q0 = fmaf(v, p01 - p00, p00), q1 = fmaf(v, p11 - p10, p10);
+    const Corners T = ldg_corners(G.te + 2 * cell);
+    const F2 P0 = fma2(w2, sub2(T.q[1], T.q[0]), T.q[0]), P1 = fma2(w2, sub2(T.q[3], T.q[2]), T.q[2]);
+    float q0, q1;
+    unpack(fma2(v2, sub2(P1, P0), P0), q0, q1);
     s.te = fmaf(u, q1 - q0, q0);
   }
   return s;

@@ -149,12 +149,14 @@ __device__ __forceinline__ Vec pair_offset(int j, const Vec& a, const Vec& b) {
 // (rn, kn).  kMixed carries the rounding of both updates in (rl, kl)
 // (Fast2Sum); the plain form leaves them at zero.  The forward kernel and the
 // adjoint's recomputation share it, so both follow the same path.
+__device__ __forceinline__ Vec chord(float h, float h2_6, const Rk4Out& o, float kx, float ky, float kz, float klx,
+                                     float kly, float klz) {
+  return {fmaf(h, kx + klx, h2_6 * o.Gx), fmaf(h, ky + kly, h2_6 * o.Gy), fmaf(h, kz + klz, h2_6 * o.Gz)};
+}
 template <bool kMixed>
-__device__ __forceinline__ void complete_step(float h, float h2_6, float h_6, const Rk4Out& o, float px, float py,
-                                              float pz, float kx, float ky, float kz, float& rlx, float& rly,
-                                              float& rlz, float& klx, float& kly, float& klz, Vec& dr, Vec& rn,
-                                              Vec& kn) {
-  dr = {fmaf(h, kx + klx, h2_6 * o.Gx), fmaf(h, ky + kly, h2_6 * o.Gy), fmaf(h, kz + klz, h2_6 * o.Gz)};
+__device__ __forceinline__ void complete_step(float h_6, const Rk4Out& o, const Vec& dr, float px, float py, float pz,
+                                              float kx, float ky, float kz, float& rlx, float& rly, float& rlz,
+                                              float& klx, float& kly, float& klz, Vec& rn, Vec& kn) {
   const Vec dk{h_6 * o.Ax, h_6 * o.Ay, h_6 * o.Az};
   if (kMixed) {
     fast_two_sum(px, dr.x + rlx, rn.x, rlx);
@@ -407,20 +409,42 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
     StagePoints sp;
     const float off_r = kCurv ? radial_reach(P.eps_reach, px, py, pz, kx, ky, kz) : 0.f;
     const Rk4Out o = rk4_central<kCurv>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.eps_reach, &sp);
-    const float kap = P.emission ? kappa_vac(o.ne1, o.te1, kap_c, ln_f) : 0.f;
+    const Vec dr = chord(h, P.h2_6, o, kx, ky, kz, klx, kly, klz);
+
+    // ---------------------------------------------- (d) ln M of step `step`
+    float lm = 0.f;
+    if constexpr (kCurv) {
+      Retrace R;
+      chord_frame(R, P.eta, P.eps_fixed, dr);
+      float c2;
+      R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
+      const bool fast = sp.clear() && c2 <= 1e-6f && R.eps <= P.eps_reach;
+      retrace_shared<NB>(P.G, slots[threadIdx.x >> 5], active && !fast, kf, h, P.h2_6, P.h2_12, px, py, pz, kx, ky, kz,
+                         R);
+      lm = R.lm;
+    } else if (NB > 0) {
+      lm = retrace_step<(NB > 0 ? NB : 4)>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky, kz, dr,
+                                           Vec{o.Gx, o.Gy, o.Gz}).lm;
+    }
+    if (!active) return;
 
     // ---------------------------------------------- (b) segment step-1 -> step
-    int stop = 0;  // TAU_STOP or STEP_LIMIT: the path ends at node `step`
+    const float kap = P.emission ? kappa_vac(o.ne1, o.te1, kap_c, ln_f) : 0.f;
     if (step >= 1) {
       const float dt = 0.5f * (kap_prev + kap) * P.hrsun;
       const float tbar = 0.5f * (te_prev + o.te1);
       const float tau0 = tau_hi + tau_lo;
       acc_add<kMixed>(tb_hi, tb_lo, tbar * one_minus_exp_neg(dt) * __expf((lns_hi + lns_lo) - tau0));
       acc_add<kMixed>(tau_hi, tau_lo, dt);
+      int stop = 0;  // TAU_STOP or STEP_LIMIT: the path ends at node `step`
       if (P.tau_stop > 0.f && tau_hi + tau_lo >= P.tau_stop) stop = kTauStop;
       else if (step >= P.max_steps) stop = kStepLimit;
+      if (stop != 0) {
+        finish(stop, px, py, pz);
+        return;
+      }
     }
-    if (active && stop == 0 && P.ckpt && (step % kCkptEvery) == 0) {
+    if (P.ckpt && (step % kCkptEvery) == 0) {
       // state at node `step` for the adjoint's recomputation: in the ray's
       // own slots, or (a tape) in the next pool slot, linked to its previous
       unsigned long long slot;
@@ -450,9 +474,8 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
     }
 
     // ---------------------------------------------- (c) complete step `step`
-    const float qx = px, qy = py, qz = pz;  // node `step` (a stopped path ends there)
-    Vec dr, rn, kn;
-    complete_step<kMixed>(h, P.h2_6, P.h_6, o, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, dr, rn, kn);
+    Vec rn, kn;
+    complete_step<kMixed>(P.h_6, o, dr, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, rn, kn);
     kap_prev = kap;
     te_prev = o.te1;
     const float rr2 = dot3(rn, rn);
@@ -460,34 +483,14 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
     if (rr2 < P.G.r_min * P.G.r_min) term = kHitInner;
     else if (rr2 > P.G.r_max * P.G.r_max && dot3(rn, kn) > 0.f) term = kExitOuter;
     else if (!isfinite(rr2 + kn.x + kn.y + kn.z)) term = kNan;
-
-    // ---------------------------------------------- (d) neighbour retrace of step `step`
-    if constexpr (kCurv) {
-      Retrace R;
-      chord_frame(R, P.eta, P.eps_fixed, dr);
-      float c2;
-      R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
-      const bool counts = stop == 0 && term != kNan;
-      const bool fast = sp.clear() && c2 <= 1e-6f && R.eps <= P.eps_reach;
-      retrace_shared<NB>(P.G, slots[threadIdx.x >> 5], active && counts && !fast, kf, h, P.h2_6,
-                                       P.h2_12, px, py, pz, kx, ky, kz, R);
-      if (counts) acc_add<kMixed>(lns_hi, lns_lo, R.lm);
-    } else if (NB > 0) {
-      const Retrace R = retrace_step<NB>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky, kz,
-                                         dr, Vec{o.Gx, o.Gy, o.Gz});
-      if (stop == 0 && term != kNan) acc_add<kMixed>(lns_hi, lns_lo, R.lm);
-    }
-    if (!active) return;
+    if (NB > 0 && term != kNan) acc_add<kMixed>(lns_hi, lns_lo, lm);
 
     // ---------------------------------------------- (e) next node, or the end of the path
-    if (stop != 0) {
-      finish(stop, qx, qy, qz);
-    } else if (term == 0) {
+    step += 1;
+    if (term == 0) {
       px = rn.x; py = rn.y; pz = rn.z;
       kx = kn.x; ky = kn.y; kz = kn.z;
-      step += 1;
     } else if (term == kNan) {
-      step += 1;
       finish(kNan, rn.x, rn.y, rn.z);
     } else {
       // clipped last segment + boundary term (Eq. 2 front to back); the
@@ -505,7 +508,6 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
       float tbc = 0.f;
       if (term == kHitInner) tbc = (P.tbc_mode == 1) ? P.tbc_K : s.te;
       if (tbc != 0.f) acc_add<kMixed>(tb_hi, tb_lo, tbc * __expf(lns - (tau_hi + tau_lo)));
-      step += 1;
       finish(term, cx, cy, cz);
     }
   };
@@ -630,8 +632,9 @@ __global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceP
       ex = px; ey = py; ez = pz;
       if (step >= 1 && P.tau_stop > 0.f && tau_hi + tau_lo >= P.tau_stop) { status = kTauStop; break; }
       if (step >= 1 && step >= P.max_steps) { status = kStepLimit; break; }
-      Vec dr, rn, kn;
-      complete_step<kMixed>(h, P.h2_6, P.h_6, o, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, dr, rn, kn);
+      const Vec dr = chord(h, P.h2_6, o, kx, ky, kz, klx, kly, klz);
+      Vec rn, kn;
+      complete_step<kMixed>(P.h_6, o, dr, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, rn, kn);
       kap_prev = kap;
       te_prev = o.te1;
       const float rr2 = dot3(rn, rn);
