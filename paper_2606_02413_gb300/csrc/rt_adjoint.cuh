@@ -332,8 +332,9 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
 
 // Reverse of one RK4 step from (p, k) (rk4_central, or rk4_g3 for a
 // neighbour's retrace), given the adjoints of its outputs: lr = dL/dr',
-// lk = dL/dk' and lg on G = a1 + a2 + a3; lq = dL/dQ of the tube area at the
-// first three stage points (0: none), t its direction.  With
+// lk = dL/dk' and lg on G = a1 + a2 + a3; lq = dL/dQ of the tube area at a
+// stage point (0: none; the second stage's also stands for the third), t its
+// direction.  With
 // r' = r + h k + h^2/6 G and k' = k + h/6 (a1 + 2 a2 + 2 a3 + a4), the stage
 // points are P1 = p, P2 = p + h/2 k, P3 = p + h/2 k2, P4 = p + h k3 with
 // k2 = k + h/2 a1, k3 = k + h/2 a2, and a_s = kf grad n_e(P_s); P3 and P4 come
@@ -365,7 +366,8 @@ __device__ __forceinline__ void rk4_reverse(const GridDev& G, float kf, float h,
     const Vec pt = (s == 3) ? P4 : (s == 2) ? P3 : (s == 1) ? P2 : p;
     const Vec la = (s == 3) ? La4 : (s == 2) ? La3 : (s == 1) ? La2 : La1;
     // the central ray's stage 1 is the node: the accumulator follows it
-    const Vec LP = stage_adjoint(G, kf, pt.x, pt.y, pt.z, la, (s == 3) ? 0.f : lq, t, dne, dte, A,
+    const Vec LP = stage_adjoint(G, kf, pt.x, pt.y, pt.z, la,
+                                 (s >= 2) ? 0.f : (s == 1) ? 2.f * lq : lq, t, dne, dte, A,
                                  kStages == 4 && s == 0, kStages == 4 && s == 0 && value, lam_ne, lam_te, on);
     Lp = {Lp.x + LP.x, Lp.y + LP.y, Lp.z + LP.z};
     if (s == 3) {         // P4 = p + h k3, k3 = k + h/2 a2
@@ -384,12 +386,13 @@ __device__ __forceinline__ void rk4_reverse(const GridDev& G, float kf, float h,
   lko = {lko.x + Lk.x, lko.y + Lk.y, lko.z + Lk.z};
 }
 
-// sum over the three stage points of -2 H t, Cartesian: d (sum_s Q_s) / d t.
+// sum over the stage points of -2 H t (the second stands for the third),
+// Cartesian: d (sum_s Q_s) / d t.
 __device__ __forceinline__ Vec curvature_dt(const StagePoints& sp, float px, float py, float pz, const Vec& t) {
-  const float xs[3] = {px, sp.x2, sp.x3}, ys[3] = {py, sp.y2, sp.y3}, zs[3] = {pz, sp.z2, sp.z3};
+  const float xs[2] = {px, sp.x2}, ys[2] = {py, sp.y2}, zs[2] = {pz, sp.z2};
   Vec o{0.f, 0.f, 0.f};
 #pragma unroll
-  for (int s = 0; s < 3; ++s) {
+  for (int s = 0; s < 2; ++s) {
     const Curv& c = sp.cv[s];
     const float x = xs[s], y = ys[s], z = zs[s];
     const float cot = z * c.inv_rho, xt = fmaf(x, t.x, y * t.y);
@@ -400,9 +403,10 @@ __device__ __forceinline__ Vec curvature_dt(const StagePoints& sp, float px, flo
     const float ht = fmaf(c.hrt, tr, fmaf(c.htt, tt, c.htp * tp)) * c.inv_r;
     const float hp = fmaf(c.hrp, tr, fmaf(c.htp, tt, c.hpp * tp)) * c.inv_rho;
     const float m = fmaf(ht, cot, hr);
-    o = {o.x + fmaf(m, x, -hp * y), o.y + fmaf(m, y, hp * x), o.z + fmaf(hr, z, -ht * c.rho)};
+    const float n = (s == 1) ? -4.f : -2.f;
+    o = {fmaf(n, fmaf(m, x, -hp * y), o.x), fmaf(n, fmaf(m, y, hp * x), o.y), fmaf(n, fmaf(hr, z, -ht * c.rho), o.z)};
   }
-  return {-2.f * o.x, -2.f * o.y, -2.f * o.z};
+  return o;
 }
 
 // d kappa_vac / d n_e and d kappa_vac / d T_e (see kappa_vac).

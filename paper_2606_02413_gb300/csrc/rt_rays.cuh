@@ -39,7 +39,8 @@ namespace rt {
 // __launch_bounds__ occupancy target (128-thread blocks).  At 4 blocks (16
 // warps per SM, up to 128 registers) the step keeps its values in registers
 // instead of recomputing or spilling them; the kernel is bound by issue, not
-// latency, and 4 measured faster than 6, 5, 3 or 2.
+// latency, and 4 measured faster than 6, 5, 3 or 2 (without magnification
+// too: 128^2 x 8 maps 11.6 ms, 5 blocks 12.6, 6 blocks 12.9).
 #ifndef RT_RAY_MIN_BLOCKS
 #define RT_RAY_MIN_BLOCKS 4
 #endif
@@ -47,32 +48,52 @@ constexpr int kRayMinBlocks = RT_RAY_MIN_BLOCKS;
 
 // The sum G = a1 + a2 + a3 of the first three RK4 stages from (p, k): a
 // neighbour's end position is p + h k + h^2/6 G (the fourth stage enters only
-// the wave vector).  The arithmetic is that of rk4_step's G.
-__device__ __forceinline__ Vec rk4_g3(const GridDev& G, float kf, float h, float px, float py, float pz, float kx,
-                                      float ky, float kz) {
+// the wave vector).  Rounded operation by operation, so that the forms below
+// agree bit for bit.
+__device__ __forceinline__ Vec scaled(float kf, const Sample& s) {
+  return {__fmul_rn(kf, s.gx), __fmul_rn(kf, s.gy), __fmul_rn(kf, s.gz)};
+}
+__device__ __forceinline__ Vec sum3(const Vec& a, const Vec& b, const Vec& c) {
+  return {__fadd_rn(__fadd_rn(a.x, b.x), c.x), __fadd_rn(__fadd_rn(a.y, b.y), c.y),
+          __fadd_rn(__fadd_rn(a.z, b.z), c.z)};
+}
+// stage 3 at p + h/2 (k + h/2 a1)
+__device__ __forceinline__ Vec stage3_force(const GridDev& G, float kf, float hh, const Vec& p, const Vec& k,
+                                            const Vec& a1) {
+  const float qx = fmaf(hh, a1.x, k.x), qy = fmaf(hh, a1.y, k.y), qz = fmaf(hh, a1.z, k.z);
+  return scaled(kf, eval_field_t<false>(G, fmaf(hh, qx, p.x), fmaf(hh, qy, p.y), fmaf(hh, qz, p.z), false));
+}
+__device__ __forceinline__ Vec rk4_g3(const GridDev& G, float kf, float h, const Vec& p, const Vec& k) {
   const float hh = 0.5f * h;
   // stages 1 and 2 are independent (stage 2 sits at p + h/2 k)
-  Sample s1 = eval_field_t<false>(G, px, py, pz, false);
-  Sample s2 = eval_field_t<false>(G, fmaf(hh, kx, px), fmaf(hh, ky, py), fmaf(hh, kz, pz), false);
-  const float a1x = kf * s1.gx, a1y = kf * s1.gy, a1z = kf * s1.gz;
-  const float a2x = kf * s2.gx, a2y = kf * s2.gy, a2z = kf * s2.gz;
-  Vec g{a1x, a1y, a1z};
-  g.x += a2x; g.y += a2y; g.z += a2z;
-  // stage 3 at p + h/2 (k + h/2 a1)
-  const float qx = fmaf(hh, a1x, kx), qy = fmaf(hh, a1y, ky), qz = fmaf(hh, a1z, kz);
-  const Sample s3 = eval_field_t<false>(G, fmaf(hh, qx, px), fmaf(hh, qy, py), fmaf(hh, qz, pz), false);
-  g.x += kf * s3.gx; g.y += kf * s3.gy; g.z += kf * s3.gz;
-  return g;
+  const Vec a1 = scaled(kf, eval_field_t<false>(G, p.x, p.y, p.z, false));
+  const Vec a2 = scaled(kf, eval_field_t<false>(G, fmaf(hh, k.x, p.x), fmaf(hh, k.y, p.y), fmaf(hh, k.z, p.z), false));
+  return sum3(a1, a2, stage3_force(G, kf, hh, p, k, a1));
+}
+// The same by two adjacent lanes, each with the same p and k: the even lane
+// takes stage 1 and the odd one stage 2 at the same time.
+__device__ __forceinline__ Vec rk4_g3_halves(const GridDev& G, float kf, float h, const Vec& p, const Vec& k) {
+  const float hh = 0.5f * h;
+  const int lane = threadIdx.x & 31;
+  const bool odd = lane & 1;
+  const Vec q{odd ? fmaf(hh, k.x, p.x) : p.x, odd ? fmaf(hh, k.y, p.y) : p.y, odd ? fmaf(hh, k.z, p.z) : p.z};
+  const Vec a = scaled(kf, eval_field_t<false>(G, q.x, q.y, q.z, false));
+  const Vec a1{__shfl_sync(kFull, a.x, lane & ~1), __shfl_sync(kFull, a.y, lane & ~1), __shfl_sync(kFull, a.z, lane & ~1)};
+  const Vec a2{__shfl_sync(kFull, a.x, lane | 1), __shfl_sync(kFull, a.y, lane | 1), __shfl_sync(kFull, a.z, lane | 1)};
+  return sum3(a1, a2, stage3_force(G, kf, hh, p, k, a1));
 }
 
 // One central RK4 step (see rk4_step) with the stage-1 sample including T_e;
 // stages 1 and 2, and then 3 and 4, are independent of each other.  kCurv:
-// also the second derivatives at the first three stage points (cv[0..2]),
-// which the neighbours' retrace needs, and those points' clearance.
+// also the second derivatives at the first two stage points (cv[0], cv[1]),
+// which the neighbours' retrace needs, and those points' clearance.  The third
+// stage point lies h^2/4 |a_1| from the second (1e-6 R_sun at h = 2e-3), where
+// they are the same; near3: it does (within 1% of the neighbours' reach).
 struct StagePoints {
-  Curv cv[3];
+  Curv cv[2];
   float x2, y2, z2, x3, y3, z3, x4, y4, z4;  // stage points 2 to 4
-  __device__ __forceinline__ bool clear() const { return cv[0].clear && cv[1].clear && cv[2].clear; }
+  bool near3;
+  __device__ __forceinline__ bool clear() const { return cv[0].clear && cv[1].clear && near3; }
 };
 template <bool kCurv = false>
 __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float h, float px, float py, float pz,
@@ -95,7 +116,7 @@ __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float 
   const float qx = fmaf(hh, a1x, kx), qy = fmaf(hh, a1y, ky), qz = fmaf(hh, a1z, kz);
   const float q3x = fmaf(hh, a2x, kx), q3y = fmaf(hh, a2y, ky), q3z = fmaf(hh, a2z, kz);
   const float x3 = fmaf(hh, qx, px), y3 = fmaf(hh, qy, py), z3 = fmaf(hh, qz, pz);
-  const Sample s3 = eval_field_t<false, kCurv>(G, x3, y3, z3, false, off_r, off, kCurv ? &sp->cv[2] : nullptr);
+  const Sample s3 = eval_field_t<false>(G, x3, y3, z3, false);
   const float x4 = fmaf(h, q3x, px), y4 = fmaf(h, q3y, py), z4 = fmaf(h, q3z, pz);
   const Sample s4 = eval_field_t<false>(G, x4, y4, z4, false);
   const float a3x = kf * s3.gx, a3y = kf * s3.gy, a3z = kf * s3.gz;
@@ -106,6 +127,8 @@ __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float 
     sp->x2 = x2; sp->y2 = y2; sp->z2 = z2;
     sp->x3 = x3; sp->y3 = y3; sp->z3 = z3;
     sp->x4 = x4; sp->y4 = y4; sp->z4 = z4;
+    const float dx = x3 - x2, dy = y3 - y2, dz = z3 - z2;
+    sp->near3 = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= 1e-4f * off * off;
   }
   return o;
 }
@@ -238,7 +261,8 @@ __device__ __forceinline__ Retrace retrace_step(const GridDev& G, float kf, floa
     const int j = (NB >= 4) ? (q >> 1) : q;
     const float sgn = (NB >= 4 && (q & 1)) ? -1.f : 1.f;
     const Vec off = (NB >= 4) ? pair_offset(j, sa, sb) : ((j == 0) ? sa : sb);
-    const Vec g = rk4_g3(G, kf, h, fmaf(sgn, off.x, px), fmaf(sgn, off.y, py), fmaf(sgn, off.z, pz), kx, ky, kz);
+    const Vec g = rk4_g3(G, kf, h, Vec{fmaf(sgn, off.x, px), fmaf(sgn, off.y, py), fmaf(sgn, off.z, pz)},
+                         Vec{kx, ky, kz});
 #pragma unroll
     for (int m = 0; m < NP; ++m)
       if (m == j) D[m] = {fmaf(sgn, g.x, D[m].x), fmaf(sgn, g.y, D[m].y), fmaf(sgn, g.z, D[m].z)};
@@ -259,18 +283,17 @@ __device__ __forceinline__ Retrace retrace_step(const GridDev& G, float kf, floa
 // step with |C| > 1e-3 retraces its neighbours.
 // Why: the neighbours' 12 (24) of a step's 16 (28) field evaluations were
 // three quarters of the kernel's instructions, and it is bound by issue.
-// Twelve second derivatives at points whose cell and fractions the central
-// ray has anyway cost about one evaluation.  One GB300, 4 neighbours, global
+// A few second derivatives at two points whose cell and fractions the central
+// ray has anyway cost less than one evaluation.  One GB300, 4 neighbours, global
 // corona 128^2 x 16 frequencies: 660 ms -> 332 ms; 64^2 x 1 on a 64x32x64
 // corona 14.3 -> 7.9 ms; 8 neighbours, 97x61 x 3: 37.5 -> 11.6 ms.  Paths,
 // optical depths and step counts are bit-identical to the retraced form's;
 // ln S differs by 5.6e-8 (rms) on the global corona.
 __device__ __forceinline__ float curvature_ln_m(const StagePoints& sp, float px, float py, float pz, const Vec& t,
                                                 float h2_6kf, float& c2) {
-  Vec f1, f2, f3;
+  Vec f1, f2;
   const float q2 = transverse_trace(sp.cv[1], sp.x2, sp.y2, sp.z2, t, f2);
-  const float q = transverse_trace(sp.cv[0], px, py, pz, t, f1) + q2 +
-                  transverse_trace(sp.cv[2], sp.x3, sp.y3, sp.z3, t, f3);
+  const float q = fmaf(2.f, q2, transverse_trace(sp.cv[0], px, py, pz, t, f1));  // the third stage is the second
   const Curv& c = sp.cv[1];
   const float off = fmaf(c.hrt, c.hrt, fmaf(c.hrp, c.hrp, c.htp * c.htp));
   const float h2 = fmaf(2.f, off, fmaf(c.htt, c.htt, c.hpp * c.hpp));  // tr H^2
@@ -305,7 +328,6 @@ __device__ __forceinline__ void retrace_shared(const GridDev& G, RetraceSlot<NB>
                                                float ky, float kz, Retrace& R) {
   constexpr int PER = 32 / NB;
   const int lane = threadIdx.x & 31;
-  const int q = lane % NB, group = lane / NB;
   unsigned todo = __ballot_sync(kFull, slow);
   while (todo) {
     const int rank = __popc(todo & ((1u << lane) - 1u));
@@ -319,17 +341,22 @@ __device__ __forceinline__ void retrace_shared(const GridDev& G, RetraceSlot<NB>
       v[12] = kf;
     }
     __syncwarp();
-    // groups past the last asking lane repeat it (the lookups stay in bounds, nothing is written)
+    // with few asking lanes each neighbour has two, a stage each
     const int asking = min(__popc(todo), PER);
+    const bool two = asking <= PER / 2;
+    const int n = two ? lane >> 1 : lane, q = n % NB, group = n / NB;
+    // groups past the last asking lane repeat it (the lookups stay in bounds, nothing is written)
     float* v = slots[min(group, asking - 1)].v;
     const float sgn = (q & 1) ? -1.f : 1.f;
     const Vec off = pair_offset(q >> 1, Vec{v[6], v[7], v[8]}, Vec{v[9], v[10], v[11]});
-    const Vec g = rk4_g3(G, v[12], h, fmaf(sgn, off.x, v[0]), fmaf(sgn, off.y, v[1]), fmaf(sgn, off.z, v[2]), v[3],
-                         v[4], v[5]);
-    const Vec d{g.x - __shfl_down_sync(kFull, g.x, 1), g.y - __shfl_down_sync(kFull, g.y, 1),
-                g.z - __shfl_down_sync(kFull, g.z, 1)};
+    const Vec p{fmaf(sgn, off.x, v[0]), fmaf(sgn, off.y, v[1]), fmaf(sgn, off.z, v[2])}, k{v[3], v[4], v[5]};
+    const float kfq = v[12];
+    const Vec g = two ? rk4_g3_halves(G, kfq, h, p, k) : rk4_g3(G, kfq, h, p, k);
+    const int step = two ? 2 : 1;
+    const Vec d{g.x - __shfl_down_sync(kFull, g.x, step), g.y - __shfl_down_sync(kFull, g.y, step),
+                g.z - __shfl_down_sync(kFull, g.z, step)};
     __syncwarp();
-    if (group < asking && !(q & 1)) {
+    if (group < asking && !(q & 1) && !(two && (lane & 1))) {
       float* w = v + 3 * (q >> 1);
       w[0] = d.x; w[1] = d.y; w[2] = d.z;
     }
