@@ -119,12 +119,6 @@ __device__ __forceinline__ Vec value_adjoint(const GridDev& G, float x, float y,
           an * c.du.z + bn * c.dv.z + cn * c.dw.z};
 }
 
-// Threads of a block of adjoint_rays: the whole SM's (see there).
-#ifndef RT_ADJ_THREADS
-#define RT_ADJ_THREADS 384
-#endif
-constexpr int kAdjThreads = RT_ADJ_THREADS;
-
 // Per-thread accumulator of the node adjoints of one cell, in shared memory
 // laid out [corner][thread] (a warp's accesses hit distinct banks): n_e's and,
 // after them, T_e's.  The adjoints of a step lie within a few 1e-3 R_sun of
@@ -132,25 +126,28 @@ constexpr int kAdjThreads = RT_ADJ_THREADS;
 // the grid with 16 atomics when the node moves to another cell or the ray
 // ends, instead of 8 or 16 per adjoint.  Stage points in another cell scatter
 // directly.
+template <int kThreadsAcc>
 struct NodeAcc {
-  float* v;    // v[q * kAdjThreads], corner q = 4 a + 2 b + c of n_e, 8 + q of T_e
+  static constexpr int T = kThreadsAcc;
+  float* v;    // v[q * T], corner q = 4 a + 2 b + c of n_e, 8 + q of T_e
   int* key;    // the cell held (-1: none)
-  int* base;   // node index of its corner (0, 0, 0)
-  int* dk1;    // k1 - k: 1, or 1 - n_phi across the phi seam
 };
 
-__device__ __forceinline__ void acc_flush(const GridDev& G, const NodeAcc& A, float* dne, float* dte) {
-  if (*A.key < 0) return;
-  const long b0 = *A.base, sr = (long)G.n_t * G.n_p;
-  const int dk = *A.dk1;
+template <int T>
+__device__ __forceinline__ void acc_flush(const GridDev& G, const NodeAcc<T>& A, float* dne, float* dte) {
+  const int cell = *A.key;
+  if (cell < 0) return;
+  // node (i, j, k) of the cell's corner (0, 0, 0): one theta row more per shell than cells
+  const long b0 = (long)cell + (long)(cell / ((G.n_t - 1) * G.n_p)) * G.n_p, sr = (long)G.n_t * G.n_p;
+  const int dk = (cell % G.n_p + 1 == G.n_p) ? 1 - G.n_p : 1;  // k1 - k: back across the phi seam
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const long id = b0 + (q >> 2) * sr + ((q >> 1) & 1) * G.n_p + (q & 1) * dk;
-    const float x = A.v[q * kAdjThreads], y = A.v[(8 + q) * kAdjThreads];
+    const float x = A.v[q * T], y = A.v[(8 + q) * T];
     if (x != 0.f) atomicAdd(dne + id, x);
     if (y != 0.f) atomicAdd(dte + id, y);
-    A.v[q * kAdjThreads] = 0.f;
-    A.v[(8 + q) * kAdjThreads] = 0.f;
+    A.v[q * T] = 0.f;
+    A.v[(8 + q) * T] = 0.f;
   }
   *A.key = -1;
 }
@@ -166,8 +163,9 @@ __device__ __forceinline__ void acc_flush(const GridDev& G, const NodeAcc& A, fl
 // lam_te) to the nodes and lam_ne grad n_e + lam_te grad T_e to the position.
 // All uses share the cell, its corners and one scatter.  on = false: a lane
 // that only keeps the warp together.
+template <int T>
 __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x, float y, float z, const Vec& lam,
-                                             float lq, const Vec& t, float* dne, float* dte, const NodeAcc& acc,
+                                             float lq, const Vec& t, float* dne, float* dte, const NodeAcc<T>& acc,
                                              bool adopt, bool value, float lam_ne, float lam_te, bool on) {
   const float rho2 = fmaf(x, x, y * y);
   const float r2 = fmaf(z, z, rho2);
@@ -271,8 +269,6 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
   if (adopt && scatter && cell != *acc.key) {
     acc_flush(G, acc, dne, dte);
     *acc.key = cell;
-    *acc.base = (i * G.n_t + j) * G.n_p + k;
-    *acc.dk1 = (k + 1 == G.n_p) ? 1 - G.n_p : 1;
   }
   float wn = 0.f;  // weight of w_c itself
   if (value) {
@@ -296,8 +292,8 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         const float uv = te ? lam_te * ((a ? u : 1.f - u) * (b ? v : 1.f - v)) : 0.f;
-        acc.v[(8 + a * 4 + b * 2) * kAdjThreads] += uv * (1.f - w);
-        acc.v[(8 + a * 4 + b * 2 + 1) * kAdjThreads] += uv * w;
+        acc.v[(8 + a * 4 + b * 2) * T] += uv * (1.f - w);
+        acc.v[(8 + a * 4 + b * 2 + 1) * T] += uv * w;
       }
   }
   const bool hit = scatter && cell == *acc.key;
@@ -316,8 +312,8 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
       const float v0 = fmaf(X, 1.f - w, -Y), v1 = fmaf(X, w, Y);
       // both branches as straight-line code: the shared adds take 0 on a
       // miss, the atomics are predicated (no divergence among the corners)
-      acc.v[(a * 4 + b * 2) * kAdjThreads] += hit ? v0 : 0.f;
-      acc.v[(a * 4 + b * 2 + 1) * kAdjThreads] += hit ? v1 : 0.f;
+      acc.v[(a * 4 + b * 2) * T] += hit ? v0 : 0.f;
+      acc.v[(a * 4 + b * 2 + 1) * T] += hit ? v1 : 0.f;
       if (miss) {
         atomicAdd(nb + a * sr + b * G.n_p, v0);
         atomicAdd(nb + a * sr + b * G.n_p + dk, v1);
@@ -343,12 +339,12 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
 // stage has no adjoint).  Adds dL/dp to lp and dL/dk to lko and scatters the
 // n_e nodes.  The stages are reversed in one loop around a single adjoint
 // (the kernel's instruction footprint, not its arithmetic, bounds it).
-template <int kStages>
+template <int kStages, int T>
 __device__ __forceinline__ void rk4_reverse(const GridDev& G, float kf, float h, const Vec& p, const Vec& k,
                                             const Vec& P3, const Vec& P4, const Vec& lr, const Vec& lk,
                                             const Vec& lg, float lq, const Vec& t, bool value, float lam_ne,
                                             float lam_te, Vec& lp, Vec& lko, float* dne, float* dte,
-                                            const NodeAcc& A, bool on) {
+                                            const NodeAcc<T>& A, bool on) {
   const float hh = 0.5f * h, h6 = h / 6.f, h3 = h / 3.f;
   const Vec P2{fmaf(hh, k.x, p.x), fmaf(hh, k.y, p.y), fmaf(hh, k.z, p.z)};
   // adjoints of the accelerations and velocities from the outputs
@@ -486,7 +482,8 @@ struct AdjointSlot {
 // derivatives here where |C| <= 1e-4, so that the first order's derivative
 // errs by less than that.
 //
-// One block holds all the warps of an SM and keeps them in the same phase (one
+// One block holds all the warps of an SM (T / 32 of them at most, see
+// launch_adjoint_rays) and keeps them in the same phase (one
 // barrier between recomputation and reverse, one per reversed step): the
 // kernel's code is larger than the instruction caches near the schedulers, and
 // warps in different phases waited 2.0 of 5.7 stall cycles per issued
@@ -498,21 +495,26 @@ struct AdjointSlot {
 // the shared retraces take about a third.  Where most lanes of a warp retrace
 // (fine grids, long steps) each takes its own neighbours: 1.0x to 1.1x of the
 // time it took before.
-template <int NB, bool kMixed>
-__global__ void __launch_bounds__(kAdjThreads, 1) adjoint_rays(const __grid_constant__ AdjParams P) {
+template <int NB, bool kMixed, int T>
+__global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ AdjParams P) {
   static_assert(NB == 0 || NB == 4, "adjoint: 4 step-wise neighbours or none");
   constexpr int K = kCkptEvery;
   constexpr int kPer = 8;  // lanes that four neighbours each fill a warp
   const int lane = threadIdx.x & 31;
   const float h = P.h;
   StepRec R[K];
-  __shared__ float acc_v[16 * kAdjThreads];
-  __shared__ int acc_key[kAdjThreads], acc_dk1[kAdjThreads], acc_base[kAdjThreads];
-  __shared__ RetraceSlot<4> fslots[kAdjThreads / 32][NB ? kPer : 1];
-  __shared__ AdjointSlot aslots[kAdjThreads / 32][NB ? kPer : 1];
-  const NodeAcc A{acc_v + threadIdx.x, acc_key + threadIdx.x, acc_base + threadIdx.x, acc_dk1 + threadIdx.x};
+  __shared__ float acc_v[16 * T];
+  __shared__ int acc_key[T];
+  // a warp's slots: the recomputation's or the reverse's
+  __shared__ union Slots {
+    RetraceSlot<4> f[NB ? kPer : 1];
+    AdjointSlot a[NB ? kPer : 1];
+    __device__ Slots() {}
+  } slots_of[T / 32];
+  Slots& S = slots_of[threadIdx.x >> 5];
+  const NodeAcc<T> A{acc_v + threadIdx.x, acc_key + threadIdx.x};
 #pragma unroll
-  for (int q = 0; q < 16; ++q) A.v[q * kAdjThreads] = 0.f;
+  for (int q = 0; q < 16; ++q) A.v[q * T] = 0.f;
   *A.key = -1;
 
   // per-ray state of the reverse sweep
@@ -630,19 +632,19 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_rays(const __grid_cons
       complete_step<kMixed>(P.h_6, o, dr, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, rn, kn);
       if (live) { rc.dr[0] = dr.x; rc.dr[1] = dr.y; rc.dr[2] = dr.z; }
       if constexpr (NB > 0) {
-        Retrace T;
-        chord_frame(T, P.eta, P.eps_fixed, dr);
+        Retrace Q;
+        chord_frame(Q, P.eta, P.eps_fixed, dr);
         float c2;
-        T.lm = curvature_ln_m(sp, px, py, pz, T.t, P.h2_6 * kf, c2);
-        const bool slow = live && !(P.curv && sp.clear() && c2 <= 1e-8f && T.eps <= P.eps_reach);
-        T.c1 = curvature_dt(sp, px, py, pz, T.t);
-        T.c2 = {0.f, 0.f, 0.f};
-        retrace_shared<NB>(P.G, fslots[threadIdx.x >> 5], slow, kf, h, P.h2_6, P.h2_12, px, py, pz, kx, ky, kz, T);
-        lns += T.lm;
+        Q.lm = curvature_ln_m(sp, px, py, pz, Q.t, P.h2_6 * kf, c2);
+        const bool slow = live && !(P.curv && sp.clear() && c2 <= 1e-8f && Q.eps <= P.eps_reach);
+        Q.c1 = curvature_dt(sp, px, py, pz, Q.t);
+        Q.c2 = {0.f, 0.f, 0.f};
+        retrace_shared<NB>(P.G, S.f, slow, kf, h, P.h2_6, P.h2_12, px, py, pz, kx, ky, kz, Q);
+        lns += Q.lm;
         if (live) {
-          rc.c1[0] = T.c1.x; rc.c1[1] = T.c1.y; rc.c1[2] = T.c1.z;
-          rc.c2[0] = T.c2.x; rc.c2[1] = T.c2.y; rc.c2[2] = T.c2.z;
-          rc.lnm = T.lm;
+          rc.c1[0] = Q.c1.x; rc.c1[1] = Q.c1.y; rc.c1[2] = Q.c1.z;
+          rc.c2[0] = Q.c2.x; rc.c2[1] = Q.c2.y; rc.c2[2] = Q.c2.z;
+          rc.lnm = Q.lm;
           rc.retraced = slow ? 1 : 0;
         }
       }
@@ -770,7 +772,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) adjoint_rays(const __grid_cons
             le = {fmaf(sn * eps, lpn.x, le.x), fmaf(sn * eps, lpn.y, le.y), fmaf(sn * eps, lpn.z, le.z)};
           };
           bool left = slow;
-          AdjointSlot* slots = aslots[threadIdx.x >> 5];
+          AdjointSlot* slots = S.a;
           // up to three passes serve 24 lanes; with more each lane takes its own
           // neighbours, whose scatters its accumulator then mostly holds
           const bool own = __popc(todo) > 3 * kPer;

@@ -1194,6 +1194,32 @@ void backward_params(rt_ctx* ctx, const rt_grid* g, const rt_view* v, const doub
   P.total = (unsigned int)((long)nf * v->nx * v->ny);
 }
 
+// One block per SM with the warps that the rays need.
+template <int NB, bool M, int T>
+cudaError_t launch_adjoint_blocks(AdjParams& A, int sm_count, cudaStream_t s) {
+  const Spread sp = spread(A.total, 32, sm_count, T / 32);
+  A.lanes = sp.lanes;
+  const int warps = (sp.warps + sm_count - 1) / sm_count;  // of a block
+  adjoint_rays<NB, M, T><<<(sp.warps + warps - 1) / warps, warps * 32, 0, s>>>(A);
+  return cudaGetLastError();
+}
+// Up to 12 warps of 168 registers or 16 of 128 (which spill a little with
+// neighbours).  A step takes a round of either about as long, 1.3 (without
+// neighbours 1.2) times for 16, and a partly filled last round from half of
+// that up, so the rounds that the rays need decide.  Measured (reverse of 8
+// maps, 12 against 16 warps, ms): 51200 rays 55 and 63, 64800 85 and 70,
+// 100352 103 and 124, 131072 137 and 130; without neighbours 26 and 28, 42 and
+// 30, 50 and 55, 68 and 57.
+template <int NB, bool M>
+cudaError_t launch_adjoint_rays(AdjParams& A, int sm_count, cudaStream_t s) {
+  auto rounds = [&](int threads) {
+    const double w = (double)A.total / ((double)threads * sm_count), full = std::floor(w);
+    return full + (w > full ? 0.5 + 0.5 * (w - full) : 0.0);
+  };
+  return rounds(512) * (NB ? 1.3 : 1.2) < rounds(384) ? launch_adjoint_blocks<NB, M, 512>(A, sm_count, s)
+                                                      : launch_adjoint_blocks<NB, M, 384>(A, sm_count, s);
+}
+
 // Zeroes the gradients and launches the reverse sweep over the checkpoints
 // (ck_off, or a tape's ck_prev / ck_last chains).
 cudaError_t launch_adjoint(rt_ctx* ctx, const rt_grid* g, const TraceParams& P, int nb, bool mixed,
@@ -1225,19 +1251,10 @@ cudaError_t launch_adjoint(rt_ctx* ctx, const rt_grid* g, const TraceParams& P, 
   A.counter = ctx->d_counter;
   A.total = P.total;
   A.mismatch = mismatch;
-  // one block of up to kAdjThreads per SM, with the warps that the rays need
-  const Spread sp = spread(P.total, 32, ctx->sm_count, kAdjThreads / 32);
-  A.lanes = sp.lanes;
-  const int warps = (sp.warps + ctx->sm_count - 1) / ctx->sm_count;  // of a block
-  const int blocks = (sp.warps + warps - 1) / warps;
-  if (nb == 0) {
-    if (mixed) adjoint_rays<0, true><<<blocks, warps * 32, 0, s>>>(A);
-    else adjoint_rays<0, false><<<blocks, warps * 32, 0, s>>>(A);
-  } else {
-    if (mixed) adjoint_rays<4, true><<<blocks, warps * 32, 0, s>>>(A);
-    else adjoint_rays<4, false><<<blocks, warps * 32, 0, s>>>(A);
-  }
-  return cudaGetLastError();
+  if (nb == 0) return mixed ? launch_adjoint_rays<0, true>(A, ctx->sm_count, s)
+                            : launch_adjoint_rays<0, false>(A, ctx->sm_count, s);
+  return mixed ? launch_adjoint_rays<4, true>(A, ctx->sm_count, s)
+               : launch_adjoint_rays<4, false>(A, ctx->sm_count, s);
 }
 
 }  // namespace

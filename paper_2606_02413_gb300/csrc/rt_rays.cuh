@@ -313,11 +313,17 @@ __device__ __forceinline__ float curvature_ln_m(const StagePoints& sp, float px,
 // The neighbours of a step that comes too near a face (about one step in
 // ten on a 64x32x64 corona at h = 2e-3, one in twenty on the global one) are
 // retraced; almost every warp has such a lane, so a branch per lane would pay
-// for all of them.  A warp's lanes retrace together the neighbours of the lanes that ask for it
-// (slow): NB lanes per asking lane, one neighbour each, 32 / NB asking lanes
-// at a time.  The arithmetic of each is retrace_step's.  Every lane of the
-// warp calls it; R.t, e1, e2, eps hold the asking lane's frame, and its ln M
-// comes back in R.lm.
+// for all of them.  A warp's lanes retrace together the neighbours of the lanes
+// that ask for it (slow): NB lanes per asking lane, one neighbour each, 32 / NB
+// asking lanes at a time; while at most half of those ask, two lanes per
+// neighbour, which take its first two stages at once (global corona 128^2 x 16:
+// 314 -> 300 ms, 40 small requests 27.1 -> 25.7 ms).  The arithmetic of each is
+// retrace_step's.  Every lane of the warp calls it; R.t, e1, e2, eps hold the
+// asking lane's frame, and its ln M comes back in R.lm.  Measured and not kept:
+// lanes that wait until a pass fills (rays that run along a face ask at every
+// step and stall: 332 -> 362 ms), and differences at the stages near a face
+// only (3% faster, but points formed in another order move ln S of single rays
+// by up to 1e-3).
 template <int NB>
 struct RetraceSlot {
   float v[(NB == 8) ? 16 : 13];  // p, k, eps e1, eps e2, kf; then D_1 ... D_{NB/2}
