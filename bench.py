@@ -39,20 +39,22 @@ R_SUN_UNITS = "R_sun"
 # Algorithmic FP32 operations (FMA = 2) of the kernel's operation list:
 # one field evaluation (radius and cell lookup, two arctangents, trilinear
 # value and three partials, Cartesian chain rule) = 111; the central ray's RK4
-# step = 4 evaluations + 60 (stage points, force scaling, G and A sums); a
-# step-wise neighbour = its seed and RK4 stages 1-3 (its end position needs
-# no fourth stage) = 3 evaluations + 36; per central step the bookkeeping
-# (tube area, basis, transfer, termination) = 120, the stage-1 T_e
-# interpolation = 15, and the neighbour-pair differences 3 per pair.
+# step = 4 evaluations + 60 (stage points, force scaling, G and A sums); the
+# tube area from the interpolant's second derivatives = 55 at each of two stage
+# points (the mixed partials, their frame components, the trace across the
+# chord, the distances to the cell's faces) + 40 (chord, second order); per
+# central step the bookkeeping (transfer, termination) = 100, the stage-1 T_e
+# interpolation = 15.  A step near a cell face retraces its neighbours as well
+# (n_nb (3 evaluations + 36), about one step in twenty on the headline
+# corona): not counted.
 FLOP_EVAL = 111
 FLOP_CENTRAL_RK4 = 60
-FLOP_NEIGHBOUR_RK4 = 36
-FLOP_STEP_BOOK = 135
+FLOP_TUBE_AREA = 2 * 55 + 40
+FLOP_STEP_BOOK = 115
 
 
 def flops_per_ray_step(n_nb: int) -> int:
-    return (4 * FLOP_EVAL + FLOP_CENTRAL_RK4 + n_nb * (3 * FLOP_EVAL + FLOP_NEIGHBOUR_RK4) + FLOP_STEP_BOOK
-            + 3 * (n_nb // 2))
+    return 4 * FLOP_EVAL + FLOP_CENTRAL_RK4 + (FLOP_TUBE_AREA if n_nb else 0) + FLOP_STEP_BOOK
 
 
 def load_peaks():

@@ -807,6 +807,8 @@ FreqDev make_freq(double f, int slab) {
 // 1.9x, 0.45 1.2x and 1.4x, 0.78 1.0x, 1.0 0.93x.  The line on the step keeps
 // eps^2, the order that the form leaves out, below 2e-5 R_sun^2, and costs
 // nothing: 64x32x64, 4 neighbours, gives 1.3x at h = 8e-3 and 0.98x at 1.6e-2.
+// An eps below 50 h^2 is small against the third stage point's distance
+// h^2/4 |a| from the second: rays with |a| = 2 would retrace (StagePoints).
 bool curvature_form(const rt_grid* g, const rt_options* o) {
   const double eps = o->eps_mode == 1 ? o->delta : o->eta * o->dtau;
   const double dth = 1.0 / g->dev.t_inv, dph = 1.0 / g->dev.p_inv;
@@ -816,7 +818,7 @@ bool curvature_form(const rt_grid* g, const rt_options* o) {
     near += w * std::min(1.0, 2.0 * eps * (0.7 / w + 1.0 / (r * dth) + 1.0 / (r * dph)));
     all += w;
   }
-  return o->dtau <= 8e-3 && near <= 0.6 * all;
+  return o->dtau <= 8e-3 && eps >= 50.0 * o->dtau * o->dtau && near <= 0.6 * all;
 }
 
 void fill_common(TraceParams& P, const rt_grid* g, const rt_options* o) {
@@ -1585,10 +1587,11 @@ rt_status rt_disk_mean_tb(const rt_view* v, const float* tb, int nf, double radi
   int cx0, cx1, cy0, cy1;
   reach(v->x0, dx, v->nx, cx0, cx1);
   reach(v->y0, dy, v->ny, cy0, cy1);
-  if (nf > (1 << 30) / kDiskCluster) return fail(RT_ERR_ARG, "rt_disk_mean_tb: nf = %d", nf);
-  disk_mean<<<nf * kDiskCluster, kDiskThreads, 0, (cudaStream_t)stream>>>(tb, v->nx, v->ny, v->x0, dx, v->y0, dy,
-                                                                         radius * radius, cx0, cx1, cy0, cy1,
-                                                                         mean_out);
+  constexpr int kMaps = (1 << 30) / kDiskCluster;  // maps of one launch
+  for (int m = 0; m < nf; m += std::min(nf - m, kMaps))
+    disk_mean<<<std::min(nf - m, kMaps) * kDiskCluster, kDiskThreads, 0, (cudaStream_t)stream>>>(
+        tb + (size_t)m * v->nx * v->ny, v->nx, v->ny, v->x0, dx, v->y0, dy, radius * radius, cx0, cx1, cy0, cy1,
+        mean_out + m);
   RT_CUDA(cudaGetLastError());
   return RT_OK;
 }
