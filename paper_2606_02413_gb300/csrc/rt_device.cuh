@@ -250,7 +250,9 @@ __device__ __forceinline__ int radial_cell(const GridDev& G, float r) {
 // derivatives, and whether the point stays clear of its cell's faces by
 // off_r radially and by off along theta and phi (off at most rho / 256: the
 // angles of an offset, and what the second derivatives leave out, are then
-// known well enough; the tests are written so that a NaN fails them).
+// known well enough; the tests are written so that a NaN fails them).  A point
+// whose fraction says nothing about its distance from the faces, in the vacuum
+// shell (u = 0, inv_dr = 0) or in the theta caps (v = 0 or 1), is never clear.
 template <bool kTe, bool kCurv = false>
 __device__ __forceinline__ Sample eval_field_t(const GridDev& G, float x, float y, float z, bool want_te,
                                                float off_r = 0.f, float off = 0.f, Curv* cv = nullptr) {
@@ -281,8 +283,8 @@ __device__ __forceinline__ Sample eval_field_t(const GridDev& G, float x, float 
   const float w = pp - (float)k;
   if (kCurv) {
     const float ot = off * inv_r, op = off * inv_rho;
-    cv->clear = fabsf(u - 0.5f) <= fmaf(-off_r, inv_dr, 0.5f) && fabsf(v - 0.5f) <= fmaf(-ot, G.t_inv, 0.5f) &&
-                fabsf(w - 0.5f) <= fmaf(-op, G.p_inv, 0.5f) && op <= 1.f / 256.f;
+    cv->clear = fabsf(u - 0.5f) < fmaf(-off_r, inv_dr, 0.5f) && fabsf(v - 0.5f) < fmaf(-ot, G.t_inv, 0.5f) &&
+                fabsf(w - 0.5f) < fmaf(-op, G.p_inv, 0.5f) && op <= 1.f / 256.f;
   }
   return sample_cell_t<kTe, kCurv>(G, i, j, k, u, v, w, tsel, inv_dr, x, y, z, inv_r, rho, inv_rho, want_te, cv);
 }
