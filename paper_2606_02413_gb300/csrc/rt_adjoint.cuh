@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ Adj
         chord_frame(Q, P.eta, P.eps_fixed, dr);
         float c2;
         Q.lm = curvature_ln_m(sp, px, py, pz, Q.t, P.h2_6 * kf, c2);
-        const bool slow = live && !(P.curv && sp.clear() && c2 <= 1e-8f && Q.eps <= P.eps_reach);
+        const bool slow = live && !(P.curv && step_clear(sp, Q, dr, P.eps_reach) && c2 <= 1e-8f);
         Q.c1 = curvature_dt(sp, px, py, pz, Q.t);
         Q.c2 = {0.f, 0.f, 0.f};
         retrace_shared<NB>(P.G, S.f, slow, kf, h, P.h2_6, P.h2_12, px, py, pz, kx, ky, kz, Q);

@@ -831,9 +831,10 @@ void fill_common(TraceParams& P, const rt_grid* g, const rt_options* o) {
   P.hrsun = (float)(h * kRsunCm);
   P.eta = (float)o->eta;
   P.eps_fixed = o->eps_mode == 1 ? (float)o->delta : 0.f;
-  // eps = eta |dr| with |dr| ~ h n, n <= 1; a step with a longer chord retraces its neighbours
+  // eps = eta |dr| with |dr| ~ h n, n <= 1; a step with a longer chord retraces its neighbours.
+  // 2% for the third stage's own shift (step_clear) and the second order along theta and phi
   P.curv = curvature_form(g, o) ? 1 : 0;
-  P.eps_reach = o->eps_mode == 1 ? (float)o->delta : (float)(1.02 * o->eta * h);
+  P.eps_reach = (float)(1.02 * (o->eps_mode == 1 ? o->delta : o->eta * h));
   P.tau_stop = (float)o->tau_stop;
   P.max_steps = o->max_steps > 0 ? o->max_steps : (int)std::ceil(40.0 * g->dev.r_max / h);
   P.tbc_mode = o->tbc_mode;

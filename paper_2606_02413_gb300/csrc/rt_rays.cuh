@@ -88,12 +88,11 @@ __device__ __forceinline__ Vec rk4_g3_halves(const GridDev& G, float kf, float h
 // also the second derivatives at the first two stage points (cv[0], cv[1]),
 // which the neighbours' retrace needs, and those points' clearance.  The third
 // stage point lies h^2/4 |a_1| from the second (1e-6 R_sun at h = 2e-3), where
-// they are the same; near3: it does (within 1% of the neighbours' reach).
+// they are the same; d3: that distance squared (step_clear looks at it).
 struct StagePoints {
   Curv cv[2];
   float x2, y2, z2, x3, y3, z3, x4, y4, z4;  // stage points 2 to 4
-  bool near3;
-  __device__ __forceinline__ bool clear() const { return cv[0].clear && cv[1].clear && near3; }
+  float d3;
 };
 template <bool kCurv = false>
 __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float h, float px, float py, float pz,
@@ -128,20 +127,24 @@ __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float 
     sp->x3 = x3; sp->y3 = y3; sp->z3 = z3;
     sp->x4 = x4; sp->y4 = y4; sp->z4 = z4;
     const float dx = x3 - x2, dy = y3 - y2, dz = z3 - z2;
-    sp->near3 = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) <= 1e-4f * off * off;
+    sp->d3 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
   }
   return o;
 }
 
 // How far a step's neighbours reach radially: they sit eps off the path
-// across the chord, so eps sin(angle of the ray to the radius), with 0.01 eps
-// for the turn of the chord and of the radius over the step (the wave vector
-// at the node stands for both) and for the second order eps^2 / 2r.
+// across the chord, so eps sin(angle of the ray to the radius), where the wave
+// vector at the node stands for the chord.  0.015 eps more covers the chord's
+// turn away from it and the third stage's shift (0.01 eps each at most, see
+// step_clear), the radius's turn over half a step and the second order
+// eps^2 / 2r; the parts never add up to more (restated in 64 bits over 40 to
+// 300 MHz, rays along and across the radius, 1e-3 to 8e-3 R_sun steps, both
+// kinds of eps).
 __device__ __forceinline__ float radial_reach(float reach, float px, float py, float pz, float kx, float ky, float kz) {
   const float pk = fmaf(px, kx, fmaf(py, ky, pz * kz));
   const float pp = fmaf(px, px, fmaf(py, py, pz * pz)), kk = fmaf(kx, kx, fmaf(ky, ky, kz * kz));
   const float c2 = __fdividef(pk * pk, pp * kk);
-  return reach * (__fsqrt_rn(fmaxf(1.f - c2, 0.f)) + 0.01f);
+  return reach * (__fsqrt_rn(fmaxf(1.f - c2, 0.f)) + 0.015f);
 }
 
 // Trace of the field's Hessian across the direction t at the point (x, y, z):
@@ -211,6 +214,21 @@ __device__ __forceinline__ void chord_frame(Retrace& R, float eta, float eps_fix
   R.t = {dr.x * ids, dr.y * ids, dr.z * ids};
   basis(R.t, R.e1, R.e2);
   R.eps = (eps_fixed > 0.f) ? eps_fixed : eta * (d2n * ids);
+}
+
+// Whether the step's neighbours stay in the cells of the stage points: these
+// are clear of the faces by `reach` (and radial_reach of it), no offset is
+// longer than that, the third stage lies within 1% of it from the second, and
+// the chord has turned from the wave vector (by about h^2/2 |a| / |dr|, twice
+// that distance over the chord) by so little that no neighbour moves by more
+// than 1%.  With eps = eta |dr| and eta <= 1/2 the last follows from the one
+// before; an offset of fixed length needs it near a turning point, where the
+// chord shrinks and the force sets its direction (without it neighbours of
+// rays near the disk centre reached up to 0.3 eps farther than allowed for).
+__device__ __forceinline__ bool step_clear(const StagePoints& sp, const Retrace& R, const Vec& dr, float reach) {
+  const float lim = 1e-4f * reach * reach;
+  return sp.cv[0].clear && sp.cv[1].clear && R.eps <= reach && sp.d3 <= lim &&
+         4.f * sp.d3 * (R.eps * R.eps) <= lim * dot3(dr, dr);
 }
 
 // c1, c2 and ln M from the raw separations D (NB >= 4: D_j = G_{+j} - G_{-j}
@@ -451,7 +469,7 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
       chord_frame(R, P.eta, P.eps_fixed, dr);
       float c2;
       R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
-      const bool fast = sp.clear() && c2 <= 1e-6f && R.eps <= P.eps_reach;
+      const bool fast = step_clear(sp, R, dr, P.eps_reach) && c2 <= 1e-6f;
       retrace_shared<NB>(P.G, slots[threadIdx.x >> 5], active && !fast, kf, h, P.h2_6, P.h2_12, px, py, pz, kx, ky, kz,
                          R);
       lm = R.lm;
@@ -683,7 +701,7 @@ __global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceP
           chord_frame(R, P.eta, P.eps_fixed, dr);
           float c2;
           R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
-          fast = sp.clear() && c2 <= 1e-6f && R.eps <= P.eps_reach;
+          fast = step_clear(sp, R, dr, P.eps_reach) && c2 <= 1e-6f;
         }
         if (!fast)
           R = retrace_step<(NB > 0 ? NB : 4)>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky,
