@@ -800,25 +800,33 @@ FreqDev make_freq(double f, int slab) {
 
 // Whether the +-pairs' tube area is taken from the field's second derivatives
 // where a step stays clear of the cells' faces (curvature_ln_m): the better
-// form while few steps come near a face.  The share that does is estimated
-// from the cells' widths, averaged over the radius: a neighbour reaches eps
-// to both sides, radially about 0.7 eps.  Measured (256^2 x 2 maps, retraced
-// over this form): share 0.05 1.7x (4 neighbours) and 2.8x (8), 0.23 1.4x and
-// 1.9x, 0.45 1.2x and 1.4x, 0.78 1.0x, 1.0 0.93x.  The line on the step keeps
-// eps^2, the order that the form leaves out, below 2e-5 R_sun^2, and costs
-// nothing: 64x32x64, 4 neighbours, gives 1.3x at h = 8e-3 and 0.98x at 1.6e-2.
-// An eps below 50 h^2 is small against the third stage point's distance
-// h^2/4 |a| from the second: rays with |a| = 2 would retrace (StagePoints).
+// form while few steps have to be retraced.  The share that does is estimated
+// over the radius, once from the cells' widths (a neighbour reaches eps to both
+// sides, radially about 0.7 eps) and once with the part of each sphere that
+// lies within 256 eps of the polar axis, where every step is retraced
+// (eval_field_t; that test, not the line on the step, bounds eps^2).  Measured,
+// 320^2 x 2 maps, time with every step retraced over this form's (4 neighbours,
+// 8 neighbours; share of faces / of both): 64x32x64 0.05 / 0.06 1.9x, 3.1x,
+// 0.24 / 0.42 1.4x, 1.6x, 0.39 / 0.68 1.09x, 1.15x, 0.48 / 0.81 0.97x, 0.98x;
+// 128x90x180 0.45 / 0.51 1.2x, 1.3x; 256x180x360 0.45 / 0.46 1.2x, 1.4x, 0.56 /
+// 0.57 1.1x, 1.25x; with faces alone 0.78 1.0x, 1.0 0.93x.  The general kernel
+// takes 1.0x to 1.07x of the former.  Steps longer than 8e-3: 64x32x64, 4
+// neighbours, 1.4x at 8e-3, 0.98x at 1.6e-2.  An eps below 50 h^2 is small
+// against the third stage point's distance h^2/4 |a| from the second: rays with
+// |a| = 2 would retrace (step_clear).
 bool curvature_form(const rt_grid* g, const rt_options* o) {
   const double eps = o->eps_mode == 1 ? o->delta : o->eta * o->dtau;
   const double dth = 1.0 / g->dev.t_inv, dph = 1.0 / g->dev.p_inv;
-  double near = 0.0, all = 0.0;
+  double faces = 0.0, both = 0.0, all = 0.0;
   for (int i = 0; i + 1 < g->n_r; ++i) {
     const double w = g->r[i + 1] - g->r[i], r = 0.5 * (g->r[i] + g->r[i + 1]);
-    near += w * std::min(1.0, 2.0 * eps * (0.7 / w + 1.0 / (r * dth) + 1.0 / (r * dph)));
+    const double f = std::min(1.0, 2.0 * eps * (0.7 / w + 1.0 / (r * dth) + 1.0 / (r * dph)));
+    const double s = std::min(1.0, 256.0 * eps / r);  // sin of the polar cap's angle
+    faces += w * f;
+    both += w * (1.0 - (1.0 - f) * std::sqrt(1.0 - s * s));
     all += w;
   }
-  return o->dtau <= 8e-3 && eps >= 50.0 * o->dtau * o->dtau && near <= 0.6 * all;
+  return o->dtau <= 8e-3 && eps >= 50.0 * o->dtau * o->dtau && faces <= 0.6 * all && both <= 0.7 * all;
 }
 
 void fill_common(TraceParams& P, const rt_grid* g, const rt_options* o) {

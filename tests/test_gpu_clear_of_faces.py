@@ -50,6 +50,7 @@ def share_of_second_derivatives(rt, ctx, grid, v, f_hz, opts):  # noqa: F811
     (4, 1.5, 1, dict(eps_mode=1, delta=5e-3)),
     (8, -0.7, 1, dict(eps_mode=1, delta=4e-3, dtau=8e-3)),
     (4, 0.3, 1, dict(eta=0.1, dtau=1.5e-3)),
+    (4, 0.3, 0, dict(eps_mode=1, delta=1e-2)),                # most of the corona lies within 256 offsets of the axis
     (4, 0.3, 0, dict(eps_mode=1, delta=2e-4)),                # small against the third stage's distance
     (4, 0.3, 0, dict(eta=0.1, dtau=8e-3)),
     (4, 0.3, 0, dict(eps_mode=1, delta=2e-2)),                # cells hardly wider than the offsets
