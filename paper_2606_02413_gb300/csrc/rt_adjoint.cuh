@@ -162,8 +162,13 @@ __device__ __forceinline__ void acc_flush(const GridDev& G, const NodeAcc<T>& A,
 // (lam_ne, lam_te) of the interpolated n_e and T_e themselves, w_c (lam_ne,
 // lam_te) to the nodes and lam_ne grad n_e + lam_te grad T_e to the position.
 // All uses share the cell, its corners and one scatter.  on = false: a lane
-// that only keeps the warp together.
-template <int T>
+// that only keeps the warp together.  kShare: the four lanes of an aligned group
+// reverse the four neighbours of one ray, acc is that ray's accumulator, and
+// what of the group falls into its cell is summed over the group before it is
+// added, two corners a lane: the parts of a +-pair nearly cancel, and must not
+// meet in other sums first (scattered by each lane on its own, n_e's gradient
+// on 5x3x4 cells was 2e-5 off, relative L2, where it is 2e-6 now).
+template <bool kShare, int T>
 __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x, float y, float z, const Vec& lam,
                                              float lq, const Vec& t, float* dne, float* dte, const NodeAcc<T>& acc,
                                              bool adopt, bool value, float lam_ne, float lam_te, bool on) {
@@ -301,6 +306,7 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
   float* nb = dne + (((long)i * G.n_t + j) * G.n_p + k);
   const long sr = (long)G.n_t * G.n_p;
   const int dk = (k + 1 == G.n_p) ? 1 - G.n_p : 1;
+  float part[8];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -312,13 +318,31 @@ __device__ __forceinline__ Vec stage_adjoint(const GridDev& G, float kf, float x
       const float v0 = fmaf(X, 1.f - w, -Y), v1 = fmaf(X, w, Y);
       // both branches as straight-line code: the shared adds take 0 on a
       // miss, the atomics are predicated (no divergence among the corners)
-      acc.v[(a * 4 + b * 2) * T] += hit ? v0 : 0.f;
-      acc.v[(a * 4 + b * 2 + 1) * T] += hit ? v1 : 0.f;
+      const int q = a * 4 + b * 2;
+      if (kShare) {
+        part[q] = hit ? v0 : 0.f;
+        part[q + 1] = hit ? v1 : 0.f;
+      } else {
+        acc.v[q * T] += hit ? v0 : 0.f;
+        acc.v[(q + 1) * T] += hit ? v1 : 0.f;
+      }
       if (miss) {
         atomicAdd(nb + a * sr + b * G.n_p, v0);
         atomicAdd(nb + a * sr + b * G.n_p + dk, v1);
       }
     }
+  if (kShare) {  // the group's sums, halved between the lanes along phi and then along theta
+    const bool c1 = threadIdx.x & 1, b1 = threadIdx.x & 2;
+    float half[4];  // corners (a, b, c1) over the pair
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+      half[n] = (c1 ? part[2 * n + 1] : part[2 * n]) + __shfl_xor_sync(kFull, c1 ? part[2 * n] : part[2 * n + 1], 1);
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const float sum = (b1 ? half[2 * a + 1] : half[2 * a]) + __shfl_xor_sync(kFull, b1 ? half[2 * a] : half[2 * a + 1], 2);
+      if (on) acc.v[(a * 4 + (threadIdx.x & 2) + (threadIdx.x & 1)) * T] += sum;
+    }
+  }
   // back to Cartesian
   const float rr = pr * inv_r, tq = pt * inv_r, pq = pf * inv_rho;
   const float h = fmaf(tq, cot, rr);
@@ -361,7 +385,7 @@ __device__ __forceinline__ void rk4_reverse(const GridDev& G, float kf, float h,
     const Vec pt = (s == 3) ? P4 : (s == 2) ? P3 : (s == 1) ? P2 : p;
     const Vec la = (s == 3) ? La4 : (s == 2) ? La3 : (s == 1) ? La2 : La1;
     // the central ray's stage 1 is the node: the accumulator follows it
-    const Vec LP = stage_adjoint(G, kf, pt.x, pt.y, pt.z, la,
+    const Vec LP = stage_adjoint<kStages == 3>(G, kf, pt.x, pt.y, pt.z, la,
                                  (s >= 2) ? 0.f : (s == 1) ? 2.f * lq : lq, t, dne, dte, A,
                                  kStages == 4 && s == 0, kStages == 4 && s == 0 && value, lam_ne, lam_te, on);
     Lp = {Lp.x + LP.x, Lp.y + LP.y, Lp.z + LP.z};
@@ -460,6 +484,7 @@ struct AdjointSlot {
       float r[3], k[3], e1[3], e2[3];  // node, wave vector, transverse basis
       float l1[3], l2[3];              // adjoints of G on the "+" member of each pair
       float eps, kf;
+      int thread;                      // the asking lane's
     } in;
     float out[4][6];                 // dL/dp, dL/dk of each neighbour
   };
@@ -492,9 +517,9 @@ struct AdjointSlot {
 // 128-thread blocks, 223 ms with the second derivatives, 173 ms with one block
 // an SM and the value adjoints in the node's own stage.  Bound by issue and
 // instruction fetch: 210 warp-instructions per ray-step (466 before), of which
-// the shared retraces take about a third.  Where most lanes of a warp retrace
-// (fine grids, long steps) each takes its own neighbours: 1.0x to 1.1x of the
-// time it took before.
+// the shared retraces take about a third.  Where every step is retraced (dtau
+// 1e-2, 64x32x64 corona, 320^2 x 2 maps) the reverse sweep takes 60 ms (75 ms
+// with a ray's neighbours one after the other in its own lane).
 template <int NB, bool kMixed, int T>
 __global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ AdjParams P) {
   static_assert(NB == 0 || NB == 4, "adjoint: 4 step-wise neighbours or none");
@@ -771,52 +796,36 @@ __global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ Adj
             Vec& le = (n < 2) ? le1 : le2;
             le = {fmaf(sn * eps, lpn.x, le.x), fmaf(sn * eps, lpn.y, le.y), fmaf(sn * eps, lpn.z, le.z)};
           };
-          bool left = slow;
           AdjointSlot* slots = S.a;
-          // up to three passes serve 24 lanes; with more each lane takes its own
-          // neighbours, whose scatters its accumulator then mostly holds
-          const bool own = __popc(todo) > 3 * kPer;
-          int q = own ? 0 : lane & 3;
-          const int group = lane >> 2;
+          const int q = lane & 3, group = lane >> 2;
+          const float sgn = (q & 1) ? -1.f : 1.f;
+          bool left = slow;
           while (todo) {
             const int rank = __popc(todo & ((1u << lane) - 1u));
-            const bool mine = left && (own || rank < kPer);
-            const float sgn = (q & 1) ? -1.f : 1.f;
-            Vec base, kk, lg;
-            float kfq;
-            bool on;
-            if (own) {
-              const Vec ev = (q < 2) ? e1 : e2, lv = (q < 2) ? lc1 : lc2;
-              const float se = sgn * eps, sl = sgn * sc;
-              base = {fmaf(se, ev.x, rr.x), fmaf(se, ev.y, rr.y), fmaf(se, ev.z, rr.z)};
-              lg = {sl * lv.x, sl * lv.y, sl * lv.z};
-              kk = rk;
-              kfq = kf;
-              on = left;
-            } else {
-              if (mine) {
-                auto& in = slots[rank].in;
-                in.r[0] = rr.x; in.r[1] = rr.y; in.r[2] = rr.z;
-                in.k[0] = rk.x; in.k[1] = rk.y; in.k[2] = rk.z;
-                in.e1[0] = e1.x; in.e1[1] = e1.y; in.e1[2] = e1.z;
-                in.e2[0] = e2.x; in.e2[1] = e2.y; in.e2[2] = e2.z;
-                in.l1[0] = sc * lc1.x; in.l1[1] = sc * lc1.y; in.l1[2] = sc * lc1.z;
-                in.l2[0] = sc * lc2.x; in.l2[1] = sc * lc2.y; in.l2[2] = sc * lc2.z;
-                in.eps = eps;
-                in.kf = kf;
-              }
-              __syncwarp();
-              const int asking = min(__popc(todo), kPer);
-              const auto& in = slots[min(group, asking - 1)].in;
-              const float* ev = (q < 2) ? in.e1 : in.e2;
-              const float* lv = (q < 2) ? in.l1 : in.l2;
-              const float se = sgn * in.eps;
-              base = {fmaf(se, ev[0], in.r[0]), fmaf(se, ev[1], in.r[1]), fmaf(se, ev[2], in.r[2])};
-              kk = {in.k[0], in.k[1], in.k[2]};
-              lg = {sgn * lv[0], sgn * lv[1], sgn * lv[2]};
-              kfq = in.kf;
-              on = group < asking;
+            const bool mine = left && rank < kPer;
+            if (mine) {
+              auto& in = slots[rank].in;
+              in.r[0] = rr.x; in.r[1] = rr.y; in.r[2] = rr.z;
+              in.k[0] = rk.x; in.k[1] = rk.y; in.k[2] = rk.z;
+              in.e1[0] = e1.x; in.e1[1] = e1.y; in.e1[2] = e1.z;
+              in.e2[0] = e2.x; in.e2[1] = e2.y; in.e2[2] = e2.z;
+              in.l1[0] = sc * lc1.x; in.l1[1] = sc * lc1.y; in.l1[2] = sc * lc1.z;
+              in.l2[0] = sc * lc2.x; in.l2[1] = sc * lc2.y; in.l2[2] = sc * lc2.z;
+              in.eps = eps;
+              in.kf = kf;
+              in.thread = threadIdx.x;
             }
+            __syncwarp();
+            // groups past the last asking lane repeat it (the lookups stay in bounds, nothing is written)
+            const int asking = min(__popc(todo), kPer);
+            const bool on = group < asking;
+            const auto& in = slots[min(group, asking - 1)].in;
+            const float* ev = (q < 2) ? in.e1 : in.e2;
+            const float* lv = (q < 2) ? in.l1 : in.l2;
+            const float se = sgn * in.eps, kfq = in.kf;
+            const Vec base{fmaf(se, ev[0], in.r[0]), fmaf(se, ev[1], in.r[1]), fmaf(se, ev[2], in.r[2])};
+            const Vec kk{in.k[0], in.k[1], in.k[2]}, lg{sgn * lv[0], sgn * lv[1], sgn * lv[2]};
+            const NodeAcc<T> Aq{acc_v + in.thread, acc_key + in.thread};
             const Vec zero{0.f, 0.f, 0.f};
             Vec lp_o = zero, lk_o = zero;
             const float hh = 0.5f * h;
@@ -824,29 +833,24 @@ __global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ Adj
             const Vec p3{fmaf(hh, fmaf(hh, kfq * s1.gx, kk.x), base.x), fmaf(hh, fmaf(hh, kfq * s1.gy, kk.y), base.y),
                          fmaf(hh, fmaf(hh, kfq * s1.gz, kk.z), base.z)};
             rk4_reverse<3>(P.G, kfq, h, base, kk, p3, zero, zero, zero, lg, 0.f, zero, false, 0.f, 0.f, lp_o, lk_o,
-                           P.dne, P.dte, A, on);
-            if (own) {
-              if (left) fold(q, lp_o, lk_o);
-              if (++q == 4) todo = 0;
-            } else {
-              __syncwarp();
-              if (on) {
-                float* out = slots[group].out[q];
-                out[0] = lp_o.x; out[1] = lp_o.y; out[2] = lp_o.z;
-                out[3] = lk_o.x; out[4] = lk_o.y; out[5] = lk_o.z;
-              }
-              __syncwarp();
-              if (mine) {
-#pragma unroll
-                for (int n = 0; n < 4; ++n) {
-                  const float* out = slots[rank].out[n];
-                  fold(n, Vec{out[0], out[1], out[2]}, Vec{out[3], out[4], out[5]});
-                }
-                left = false;
-              }
-              __syncwarp();  // the slots are read: the next lanes may fill them
-              todo = __ballot_sync(kFull, left);
+                           P.dne, P.dte, Aq, on);
+            __syncwarp();
+            if (on) {
+              float* out = slots[group].out[q];
+              out[0] = lp_o.x; out[1] = lp_o.y; out[2] = lp_o.z;
+              out[3] = lk_o.x; out[4] = lk_o.y; out[5] = lk_o.z;
             }
+            __syncwarp();
+            if (mine) {
+#pragma unroll
+              for (int n = 0; n < 4; ++n) {
+                const float* out = slots[rank].out[n];
+                fold(n, Vec{out[0], out[1], out[2]}, Vec{out[3], out[4], out[5]});
+              }
+              left = false;
+            }
+            __syncwarp();  // the slots are read: the next lanes may fill them
+            todo = __ballot_sync(kFull, left);
           }
           if (slow) {
             lt = {lm1 * (c1.y * c2.z - c1.z * c2.y), lm1 * (c1.z * c2.x - c1.x * c2.z),
