@@ -751,6 +751,7 @@ __global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ Adj
     for (int it = 0; any(active && it < n_s); ++it) {
       const int t = n_s - 1 - it;
       const bool stepping = active && t >= 0;
+      if (!__any_sync(kFull, stepping)) continue;  // a warp that waits for the block's others leaves them the SM
       const StepRec rc = R[max(t, 0)];
       const bool clip = last_seg && it == 0 && clipped;
 

@@ -64,3 +64,21 @@ def test_full_warps(rt, ctx, shape, nx, ny, opts):  # noqa: F811
     rel = [np.linalg.norm(a - b) / np.linalg.norm(b) for a, b in zip(whole, parts)]
     print(shape, opts, "relative L2", rel)
     assert max(rel) <= 2e-5, rel
+
+
+@pytest.mark.parametrize("opts", [dict(dtau=4e-3), dict(dtau=8e-3, s_mode=2)])
+def test_few_weights(rt, ctx, opts):  # noqa: F811
+    """Three weighted rays in a view of 20480: most warps of their blocks have
+    nothing to do at any step.  Against the single rays (as test_full_warps)."""
+    grid = ctx.load(corona(24, 16, 32))
+    d = 2.0 ** -6
+    pix = [(3, 5, 1.0), (80, 64, -2.0), (159, 127, 0.5)]
+    w = np.zeros((1, 128, 160))
+    parts = [0.0, 0.0]
+    for ix, iy, c in pix:
+        w[0, iy, ix] = c
+        v = cs.View(0.3, 0.25, 1, 1, -1.25 + ix * d, -1.25 + (ix + 1) * d, -1.0 + iy * d, -1.0 + (iy + 1) * d)
+        parts = [a + b for a, b in zip(parts, gradient(rt, ctx, grid, v, [90e6], np.full((1, 1, 1), c), opts))]
+    whole = gradient(rt, ctx, grid, cs.View(0.3, 0.25, 160, 128, -1.25, 1.25, -1.0, 1.0), [90e6], w, opts)
+    for a, b in zip(whole, parts):
+        assert np.linalg.norm(a - b) <= 2e-5 * np.linalg.norm(b)
