@@ -432,17 +432,21 @@ cudaError_t launch_rays(const TraceParams& P, int sm_count, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// the path recorder in the form trace_rays takes, so that both agree bit for bit
+// the path recorder in the form trace_rays takes, so that both agree bit for
+// bit, with its rays spread over the schedulers (kPathWarps: the warps of an SM
+// at up to 128 registers)
+constexpr int kPathWarps = 16;
 template <int NB, bool M>
 void launch_paths(const TraceParams& P, const int* pix, int n, int cap, PathNode* path, int* count, float* tb,
-                  RayDiag* diag, int blocks, cudaStream_t s) {
+                  RayDiag* diag, cudaStream_t s) {
+  const int rays = P.lanes * (kPathThreads / 32), blocks = (n + rays - 1) / rays;
   if constexpr (NB >= 4) {
     if (P.curv) {
-      trace_paths<NB, M, true><<<blocks, 64, 0, s>>>(P, pix, n, cap, path, count, tb, diag);
+      trace_paths<NB, M, true><<<blocks, kPathThreads, 0, s>>>(P, pix, n, cap, path, count, tb, diag);
       return;
     }
   }
-  trace_paths<NB, M, false><<<blocks, 64, 0, s>>>(P, pix, n, cap, path, count, tb, diag);
+  trace_paths<NB, M, false><<<blocks, kPathThreads, 0, s>>>(P, pix, n, cap, path, count, tb, diag);
 }
 
 // nb: neighbour rays per bundle (0 = magnification off); tube: persistent
@@ -1519,12 +1523,12 @@ rt_status rt_trace_paths(rt_ctx* ctx, const rt_grid* g, const rt_view* v, double
   cudaError_t e = cudaMemcpyAsync(d_pix, pixels, sizeof(int) * n, cudaMemcpyHostToDevice, s);
   PathNode* pn = reinterpret_cast<PathNode*>(nodes);
   RayDiag* dg = reinterpret_cast<RayDiag*>(diag);
-  const int blocks = (n + 63) / 64;
+  P.lanes = spread((unsigned)n, 32, ctx->sm_count, kPathWarps).lanes;
   const bool mixed = o->precision == RT_MIXED;
   if (e == cudaSuccess) {
 #define RT_PATHS(NB)                                                                          \
-    (mixed ? launch_paths<NB, true>(P, d_pix, n, cap, pn, n_nodes, tb_out, dg, blocks, s) \
-           : launch_paths<NB, false>(P, d_pix, n, cap, pn, n_nodes, tb_out, dg, blocks, s))
+    (mixed ? launch_paths<NB, true>(P, d_pix, n, cap, pn, n_nodes, tb_out, dg, s) \
+           : launch_paths<NB, false>(P, d_pix, n, cap, pn, n_nodes, tb_out, dg, s))
     switch (nb) {
       case 0: RT_PATHS(0); break;
       case 2: RT_PATHS(2); break;

@@ -635,15 +635,22 @@ struct PathNode {
 
 // Ray-fan diagnostics (Sec. 3.2, Figs. 4 and 6): the rays of the given pixels
 // at one frequency, one thread each, stepped exactly as trace_rays steps
-// them (the same step code in the same order), recording every node.
+// them (the same step code in the same order), recording every node.  A warp
+// takes P.lanes rays (as few as fill the schedulers): where one lane retraces
+// its neighbours the warp's others wait.  One GB300, 64x32x64 corona, 16, 256
+// and 4096 rays with 4 neighbours: 9.5, 10.9 and 23.1 ms with full warps and
+// every neighbour retraced, 4.7, 6.2 and 19.9 ms so.
 // The first `cap` nodes of ray i go to path[i * cap ...], its node count to
 // count[i], and its T_b and diagnostics to tb[i] and diag[i].
+constexpr int kPathThreads = 64;
 template <int NB, bool kMixed, bool kCurv>
-__global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceParams P, const int* __restrict__ pix,
-                                                  int n, int cap, PathNode* __restrict__ path, int* __restrict__ count,
-                                                  float* __restrict__ tb, RayDiag* __restrict__ diag) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+__global__ void __launch_bounds__(kPathThreads)
+    trace_paths(const __grid_constant__ TraceParams P, const int* __restrict__ pix, int n, int cap,
+                PathNode* __restrict__ path, int* __restrict__ count, float* __restrict__ tb,
+                RayDiag* __restrict__ diag) {
+  const int lane = threadIdx.x & 31;
+  const int i = (blockIdx.x * (kPathThreads / 32) + (threadIdx.x >> 5)) * P.lanes + lane;
+  if (lane >= P.lanes || i >= n) return;
   const float h = P.h;
   RayStart rs;
   rs.V = &P.view;
@@ -671,6 +678,27 @@ __global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceP
       StagePoints sp;
       const float off_r = kCurv ? radial_reach(P.eps_reach, px, py, pz, kx, ky, kz) : 0.f;
       const Rk4Out o = rk4_central<kCurv>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.eps_reach, &sp);
+      // the step's end and ln M before the transfer, as in trace_rays: neither
+      // waits for its exponentials (256 rays, 4 neighbours: 6.35 -> 6.17 ms)
+      const Vec dr = chord(h, P.h2_6, o, kx, ky, kz, klx, kly, klz);
+      Vec rn, kn;
+      complete_step<kMixed>(P.h_6, o, dr, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, rn, kn);
+      const float rr2 = dot3(rn, rn);
+      float lm = 0.f;
+      if (NB > 0) {
+        Retrace R;
+        bool fast = false;
+        if (kCurv) {
+          chord_frame(R, P.eta, P.eps_fixed, dr);
+          float c2;
+          R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
+          fast = step_clear(sp, R, dr, P.eps_reach) && c2 <= 1e-6f;
+        }
+        if (!fast)
+          R = retrace_step<(NB > 0 ? NB : 4)>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky,
+                                              kz, dr, Vec{o.Gx, o.Gy, o.Gz});
+        lm = R.lm;
+      }
       const float kap = P.emission ? kappa_vac(o.ne1, o.te1, kap_c, ln_f) : 0.f;
       if (step >= 1) {
         const float dt = 0.5f * (kap_prev + kap) * P.hrsun;
@@ -683,31 +711,16 @@ __global__ void __launch_bounds__(64) trace_paths(const __grid_constant__ TraceP
       ex = px; ey = py; ez = pz;
       if (step >= 1 && P.tau_stop > 0.f && tau_hi + tau_lo >= P.tau_stop) { status = kTauStop; break; }
       if (step >= 1 && step >= P.max_steps) { status = kStepLimit; break; }
-      const Vec dr = chord(h, P.h2_6, o, kx, ky, kz, klx, kly, klz);
-      Vec rn, kn;
-      complete_step<kMixed>(P.h_6, o, dr, px, py, pz, kx, ky, kz, rlx, rly, rlz, klx, kly, klz, rn, kn);
       kap_prev = kap;
       te_prev = o.te1;
-      const float rr2 = dot3(rn, rn);
       int term = 0;
       if (rr2 < P.G.r_min * P.G.r_min) term = kHitInner;
       else if (rr2 > P.G.r_max * P.G.r_max && dot3(rn, kn) > 0.f) term = kExitOuter;
       else if (!isfinite(rr2 + kn.x + kn.y + kn.z)) term = kNan;
       dls = 0.f;
       if (NB > 0 && term != kNan) {
-        Retrace R;
-        bool fast = false;
-        if (kCurv) {
-          chord_frame(R, P.eta, P.eps_fixed, dr);
-          float c2;
-          R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
-          fast = step_clear(sp, R, dr, P.eps_reach) && c2 <= 1e-6f;
-        }
-        if (!fast)
-          R = retrace_step<(NB > 0 ? NB : 4)>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky,
-                                              kz, dr, Vec{o.Gx, o.Gy, o.Gz});
-        acc_add<kMixed>(lns_hi, lns_lo, R.lm);
-        dls = R.lm * rsqrtf(dot3(dr, dr));
+        acc_add<kMixed>(lns_hi, lns_lo, lm);
+        dls = lm * rsqrtf(dot3(dr, dr));
       }
       if (term == 0) {
         px = rn.x; py = rn.y; pz = rn.z;
