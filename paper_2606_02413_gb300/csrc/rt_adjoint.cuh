@@ -29,9 +29,8 @@ namespace rt {
 // --------------------------------------------------------- cell geometry
 struct CellGeom {
   int i, j, k, k1;           // cell and wrapped phi neighbour
-  float u, v, w, tsel;       // fractions; tsel = 0 in the clamped theta caps
-  Vec du, dv, dw;            // Cartesian gradients of u, v, w
-  float inv_r, rho, inv_rho; // 1 / |x|, distance from the z axis and its inverse (0 on the axis)
+  float u, v, w;             // fractions
+  Vec du, dv, dw;            // Cartesian gradients of u, v, w (dv = 0 in the clamped theta caps)
   bool vac;                  // beyond the outer band
 };
 
@@ -44,9 +43,8 @@ __device__ __forceinline__ CellGeom cell_geom(const GridDev& G, float x, float y
   c.vac = !(r <= G.r_vac);
   if (c.vac) {
     c.i = c.j = c.k = c.k1 = 0;
-    c.u = c.v = c.w = c.tsel = 0.f;
+    c.u = c.v = c.w = 0.f;
     c.du = c.dv = c.dw = {0.f, 0.f, 0.f};
-    c.inv_r = c.rho = c.inv_rho = 0.f;
     return c;
   }
   float2 rc;
@@ -54,15 +52,12 @@ __device__ __forceinline__ CellGeom cell_geom(const GridDev& G, float x, float y
   c.u = (r - rc.x) * rc.y;
   const float inv_rho = (rho2 > 0.f) ? rsqrtf(rho2) : 0.f;
   const float rho = rho2 * inv_rho;
-  c.inv_r = inv_r;
-  c.rho = rho;
-  c.inv_rho = inv_rho;
   // theta cell as in the field evaluation: clamped to the outermost cells,
   // where the fraction sticks at 0 or 1 and the theta derivative is off
   const float tt = (atan2_grid<true>(rho, z) - G.t0) * G.t_inv;
   c.j = min(max(__float2int_rd(tt), 0), G.n_t - 2);
   c.v = fminf(fmaxf(tt - (float)c.j, 0.f), 1.f);
-  c.tsel = (tt > 0.f && tt < G.t_last) ? 1.f : 0.f;
+  const float tsel = (tt > 0.f && tt < G.t_last) ? 1.f : 0.f;
   float ph = atan2_grid(y, x) - G.p0;
   if (ph < 0.f) ph += kTwoPiF;
   if (ph >= kTwoPiF) ph -= kTwoPiF;
@@ -74,7 +69,7 @@ __device__ __forceinline__ CellGeom cell_geom(const GridDev& G, float x, float y
   const float a = rc.y * inv_r;
   c.du = {a * x, a * y, a * z};
   const float ir2 = inv_r * inv_r;
-  const float bt = c.tsel * G.t_inv * ir2;
+  const float bt = tsel * G.t_inv * ir2;
   c.dv = {bt * z * x * inv_rho, bt * z * y * inv_rho, -bt * rho};
   const float bp = G.p_inv * inv_rho * inv_rho;
   c.dw = {-bp * y, bp * x, 0.f};

@@ -240,11 +240,6 @@ __device__ __forceinline__ int radial_lookup(const GridDev& G, float r, float& R
   return __float_as_int(base) + (up ? 1 : 0);
 }
 
-__device__ __forceinline__ int radial_cell(const GridDev& G, float r) {
-  float R, inv;
-  return radial_lookup(G, r, R, inv);
-}
-
 // The field at (x, y, z): trilinear n_e (and T_e when kTe and want_te) and
 // the exact gradient of the n_e interpolant.  kCurv: also its second
 // derivatives, and whether the point stays clear of its cell's faces by
@@ -551,26 +546,6 @@ __device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& 
   s = a + b;
   e = b - (s - a);
 }
-
-// Running sum.  kComp = true keeps the rounding error of every addition
-// (TwoSum) and carries it, so 10^4-term sums stay near double precision;
-// kComp = false is the plain FP32 sum.
-template <bool kComp>
-struct Acc {
-  float hi, lo;
-  __device__ __forceinline__ void zero() { hi = 0.f; lo = 0.f; }
-  __device__ __forceinline__ void add(float x) {
-    if (kComp) {
-      float s, e;
-      two_sum(hi, x, s, e);
-      hi = s;
-      lo += e;
-    } else {
-      hi += x;
-    }
-  }
-  __device__ __forceinline__ float val() const { return kComp ? hi + lo : hi; }
-};
 
 // -------------------------------------------------------- kernel params
 struct RayDiag {
