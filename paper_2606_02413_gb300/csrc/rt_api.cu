@@ -366,12 +366,12 @@ __global__ void __cluster_dims__(kDiskCluster, 1, 1) __launch_bounds__(kDiskThre
   }
 }
 
-template <int NB, bool M, bool T>
-int blocks_per_sm() {
+template <int NB, bool M>
+int tube_blocks_per_sm() {
   static int cached = -1;
   if (cached < 0) {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, trace_bundles<NB, M, T>, kThreads, 0) != cudaSuccess || b < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, trace_bundles<NB, M>, kThreads, 0) != cudaSuccess || b < 1)
       b = 1;
     cached = b;
   }
@@ -414,12 +414,12 @@ Spread spread(unsigned total, int per_warp, int sm_count, int warps_per_sm) {
 // tube mode: the lane-parallel bundle kernel (persistent neighbours)
 template <int NB, bool M>
 cudaError_t launch_tube(const TraceParams& P, int sm_count, cudaStream_t s) {
-  const int fit = blocks_per_sm<NB, M, true>();
+  const int fit = tube_blocks_per_sm<NB, M>();
   const int per_sm = (P.blocks_per_sm > 0) ? std::min(P.blocks_per_sm, fit) : fit;
   const Spread sp = spread(P.total, 32 / (NB + 1), sm_count, per_sm * (kThreads / 32));
   TraceParams Q = P;
   Q.lanes = sp.lanes;
-  trace_bundles<NB, M, true><<<(sp.warps * 32 + kThreads - 1) / kThreads, kThreads, 0, s>>>(Q);
+  trace_bundles<NB, M><<<(sp.warps * 32 + kThreads - 1) / kThreads, kThreads, 0, s>>>(Q);
   return cudaGetLastError();
 }
 

@@ -1,25 +1,25 @@
-// The persistent warp-cooperative ray-bundle kernel.
+// Ray launch and vector helpers shared by every kernel, and the
+// warp-cooperative ray-bundle kernel of tube mode.
 //
-// One bundle = the central ray of a (pixel, frequency) plus NB step-wise
-// neighbour rays (Sec. 2.1, Eqs. 5-11) on NB + 1 adjacent lanes; 32 / (NB+1)
-// bundles share a warp.  The neighbours of step i can only start once the
-// central step i is known (they need its chord t^i, Eqs. 5-8), so the two are
-// pipelined: in every iteration the central lane takes step i while its
-// neighbours retrace step i - 1, and the magnification M^i and the transfer
-// of segment i - 1 are settled at the end of that iteration.
+// One bundle = the central ray of a (pixel, frequency) plus NB persistent
+// neighbour rays (Sec. 2.1, Eqs. 9-11 along the whole path) on NB + 1 adjacent
+// lanes; 32 / (NB+1) bundles share a warp.  The neighbours step in lock-step
+// with the central ray, and the magnification and the transfer of a segment
+// are settled on the central lane at the end of each iteration.
 //
-// Precision (template kMixed):
-//   - neighbour separations are never formed as differences of absolute
-//     positions.  A neighbour started at r^i + s eps e with the central k^i
-//     ends at r^i + s eps e + h k^i + h^2/6 G_s, so the central difference
-//     of a +-e pair is d = eps e + h^2/12 (G_+ - G_-) exactly, and with
-//     c_j = (d_j - eps e_j) / eps,
-//       |det[d1, d2, t]| / eps^2 = |1 + c1.e1 + c2.e2 + t.(c1 x c2)|
-//     for the orthonormal right-handed (e1, e2, t).  ln M = log1p of that.
-//   - kMixed keeps the central position / wave vector and the tau, ln S, T_b
-//     sums as compensated float pairs (TwoSum), which holds them near double
-//     precision over 10^4-step rays at FP32 instruction cost (FP64 runs at
-//     a small fraction of the FP32 rate on this GPU).
+// Precision (template kMixed): the central position / wave vector and the tau
+// and T_b sums are kept as compensated float pairs (TwoSum), which holds them
+// near double precision over 10^4-step rays at FP32 instruction cost (FP64 runs
+// at a small fraction of the FP32 rate on this GPU); the neighbours' offsets
+// carry the rounding of their increments.
+//
+// Step-wise magnification (rt_rays.cuh) never forms a separation as the
+// difference of absolute positions either.  A neighbour started at
+// r^i + s eps e with the central k^i ends at r^i + s eps e + h k^i + h^2/6 G_s,
+// so the central difference of a +-e pair is d = eps e + h^2/12 (G_+ - G_-)
+// exactly, and with c_j = (d_j - eps e_j) / eps,
+//   |det[d1, d2, t]| / eps^2 = |1 + c1.e1 + c2.e2 + t.(c1 x c2)|
+// for the orthonormal right-handed (e1, e2, t).  ln M = log1p of that.
 //
 // Work distribution: each bundle takes a ticket from a global atomic queue
 // when it finishes (warp-aggregated), so rays of very uneven length keep
@@ -48,16 +48,11 @@ __device__ __forceinline__ void basis(const Vec& t, Vec& e1, Vec& e2) {
   e2 = {t.y * e1.z - t.z * e1.y, t.z * e1.x - t.x * e1.z, t.x * e1.y - t.y * e1.x};
 }
 
-// c1.e1 + c2.e2 + t.(c1 x c2) = M - 1 (see the file comment), and ln |M|.
+// c1.e1 + c2.e2 + t.(c1 x c2) = M - 1 (see the file comment).
 __device__ __forceinline__ float tube_m1(const Vec& c1, const Vec& c2, const Vec& e1, const Vec& e2,
                                          const Vec& t) {
   const float cx = c1.y * c2.z - c1.z * c2.y, cy = c1.z * c2.x - c1.x * c2.z, cz = c1.x * c2.y - c1.y * c2.x;
   return dot3(c1, e1) + dot3(c2, e2) + fmaf(t.x, cx, fmaf(t.y, cy, t.z * cz));
-}
-
-__device__ __forceinline__ float ln_m(const Vec& c1, const Vec& c2, const Vec& e1, const Vec& e2,
-                                      const Vec& t) {
-  return log1p_small(tube_m1(c1, c2, e1, e2, t));
 }
 
 // Root alpha in [0, 1] of |r + alpha dr| = R on the chord (stable form).
@@ -171,7 +166,6 @@ __device__ __forceinline__ RayStart start_ray(const TraceParams& P, unsigned int
 // Per-bundle state of the central lane, kept in shared memory so that only
 // the RK4 state lives in registers across the four field evaluations.
 struct BundleState {
-  unsigned int item;                                    // ticket of this ray
   float* out;                                           // T_b of this ray
   RayDiag* dg;                                          // its diagnostics or null
   int step, status;
@@ -179,10 +173,8 @@ struct BundleState {
   float tau_hi, tau_lo, lns_hi, lns_lo, tb_hi, tb_lo;  // running sums (lo: compensation)
   float rl[3], kl[3];                                   // compensation of r and k
   float kap_prev, te_prev;                              // node i-1 transfer values
-  float t[3], e1[3], e2[3], eps;                        // basis of the retraced step
-  float g0[3];                                          // central G of that step (2 neighbours)
   float alpha, pc[3];                                   // clipped last step
-  // tube mode: launch data the neighbour lanes read to start their rays
+  // launch data the neighbour lanes read to start their rays
   const ViewDev* view;
   float u, v, sc, nc, nec, kn2;
   int tube_ok;
@@ -223,13 +215,13 @@ __device__ __forceinline__ void acc_add(float& hi, float& lo, float x) {
   }
 }
 
-// kTube: the neighbours are persistent rays launched at image-plane offsets
+// Tube mode: the neighbours are persistent rays launched at image-plane offsets
 // +-delta and integrated in lock-step with the central ray; each neighbour
 // lane carries its offset (dr, dk) from the central ray, updated with the
 // difference of RK4 increments, and S = |det[d1, d2, t]| is taken after every
 // step with central differences d_j of those offsets (S_0 = delta^2).
-template <int NB, bool kMixed, bool kTube>
-__global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks) trace_bundles(const __grid_constant__ TraceParams P) {
+template <int NB, bool kMixed>
+__global__ void __launch_bounds__(kThreads, kMinBlocksTube) trace_bundles(const __grid_constant__ TraceParams P) {
   constexpr int L = NB + 1;
   constexpr int BPW = 32 / L;
   __shared__ BundleState S[kThreads / 32][BPW];
@@ -245,14 +237,13 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
     B.steps_done = 0;
     B.rays_done = 0;
   }
-  // ---- per-lane RK4 start state (central: its node; neighbour: its seed)
+  // ---- per-lane RK4 start state (central: its node; neighbour: its offset from it)
   float px = 0.f, py = 0.f, pz = 0.f, kx = 0.f, ky = 0.f, kz = 0.f;
-  bool has_seed = false;  // neighbour lanes: a retrace is pending
+  bool entered = false;  // neighbour lanes: the ray entered the corona
   int phase = 0;          // central: 0 needs work, 1 stepping, 2 final (clipped) segment
-  bool emitted = false;   // central: its neighbours retrace a step this iteration
   bool exhausted = !central || lane / L >= P.lanes;
-  bool fresh = false;     // central (tube mode): a ray started in this iteration
-  // tube neighbours (mixed form): rounding carried by the offset accumulation
+  bool fresh = false;     // central: a ray started in this iteration
+  // neighbours (mixed form): rounding carried by the offset accumulation
   float lpx = 0.f, lpy = 0.f, lpz = 0.f, lkx = 0.f, lky = 0.f, lkz = 0.f;
 
   auto finish = [&](int st, float ex, float ey, float ez, float tb_val) {
@@ -290,14 +281,12 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
           B.out = rs.out;
           B.dg = rs.dg;
           if (rs.valid) {  // a ragged chunk tail has no ray behind the ticket: take another
-            B.item = item;
             B.kf = P.straight ? 0.f : rs.F->kf;
             B.kap_c = rs.F->kap_c;
             B.ln_f = rs.F->ln_f;
             B.step = 0;
             B.tau_hi = B.tau_lo = B.lns_hi = B.lns_lo = B.tb_hi = B.tb_lo = 0.f;
             B.rl[0] = B.rl[1] = B.rl[2] = B.kl[0] = B.kl[1] = B.kl[2] = 0.f;
-            emitted = false;
             if (!rs.enter) {
               finish(kMiss, rs.px, rs.py, rs.pz, 0.f);
             } else {
@@ -305,15 +294,13 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
               kx = rs.kx; ky = rs.ky; kz = rs.kz;
               phase = 1;
               need = false;
-              if (kTube) {
-                B.view = rs.V;
-                B.u = rs.u; B.v = rs.v;
-                B.sc = rs.sc;
-                B.nc = rs.nc;
-                B.nec = rs.nec;
-                B.kn2 = rs.F->kn2;
-                fresh = true;
-              }
+              B.view = rs.V;
+              B.u = rs.u; B.v = rs.v;
+              B.sc = rs.sc;
+              B.nc = rs.nc;
+              B.nec = rs.nec;
+              B.kn2 = rs.F->kn2;
+              fresh = true;
             }
           }
         }
@@ -322,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
     }
     if (!__any_sync(kFull, phase != 0)) break;
 
-    if (kTube) {
+    {
       // neighbours of a new bundle launch from their offset pixel positions:
       // entry offsets and wave-vector offsets formed without cancellation
       const bool fr = __shfl_sync(kFull, fresh ? 1 : 0, base) != 0;
@@ -359,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
             kx = ky = kz = 0.f;
           }
         }
-        has_seed = ok;
+        entered = ok;
       }
       const unsigned okmask = __ballot_sync(kFull, ok);
       if (central && fresh) {
@@ -370,15 +357,15 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
     }
 
     // ------------------------------------------------------------ RK4
-    // central lanes step (phase 1); neighbour lanes retrace (has_seed), or
-    // in tube mode step their own rays from the central state + offsets
+    // central lanes step (phase 1), neighbour lanes their own rays from the
+    // central state + offsets
     const float kf_lane = __shfl_sync(kFull, (central && phase != 0) ? B.kf : 0.f, base);
     const int bphase = __shfl_sync(kFull, phase, base);
-    const bool work = central ? (phase == 1) : (kTube ? (has_seed && bphase == 1) : has_seed);
+    const bool work = central ? (phase == 1) : (entered && bphase == 1);
     Rk4Out o;
     o.Gx = o.Gy = o.Gz = o.Ax = o.Ay = o.Az = 0.f;
     o.ne1 = o.te1 = 0.f;
-    if (kTube) {
+    {
       // every ray of the bundle steps about the central node (b, its low part l)
       float lx = 0.f, ly = 0.f, lz = 0.f;
       if (kMixed && central) { lx = B.rl[0]; ly = B.rl[1]; lz = B.rl[2]; }
@@ -392,8 +379,6 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
         o = rk4_step_base(P.G, kf_lane, h, bp, lx, ly, lz, ckx, cky, ckz, central ? 0.f : px, central ? 0.f : py,
                           central ? 0.f : pz, central ? 0.f : kx, central ? 0.f : ky, central ? 0.f : kz, central);
       }
-    } else if (work) {
-      o = rk4_step(P.G, kf_lane, h, px, py, pz, kx, ky, kz, central);
     }
     if (central && phase == 2) {  // the clip point closes the path
       const Sample s = eval_field(P.G, B.pc[0], B.pc[1], B.pc[2], true);
@@ -402,10 +387,9 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
     }
 
     // ------------------------------------------------- neighbour exchange
-    // raw separations: NB >= 4: D_j = G_{+j} - G_{-j}; NB == 2: G_j
-    // (tube mode: the offsets after this step; central differences for 4, 8)
+    // the offsets after this step (central differences for 4, 8)
     Vec d1{0.f, 0.f, 0.f}, d2{0.f, 0.f, 0.f}, d3{0.f, 0.f, 0.f}, d4{0.f, 0.f, 0.f};
-    if (kTube) {
+    {
       const float gcx = __shfl_sync(kFull, o.Gx, base), gcy = __shfl_sync(kFull, o.Gy, base),
                   gcz = __shfl_sync(kFull, o.Gz, base);
       const float acx = __shfl_sync(kFull, o.Ax, base), acy = __shfl_sync(kFull, o.Ay, base),
@@ -443,51 +427,10 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
           d4 = {__shfl_sync(kFull, dx, base + 7), __shfl_sync(kFull, dy, base + 7), __shfl_sync(kFull, dz, base + 7)};
         }
       }
-    } else if (NB == 2) {
-      d1 = {__shfl_sync(kFull, o.Gx, base + 1), __shfl_sync(kFull, o.Gy, base + 1), __shfl_sync(kFull, o.Gz, base + 1)};
-      d2 = {__shfl_sync(kFull, o.Gx, base + 2), __shfl_sync(kFull, o.Gy, base + 2), __shfl_sync(kFull, o.Gz, base + 2)};
-    } else if (NB >= 4) {
-      // "+" members (odd roles) form G_+ - G_- with their "-" partner
-      const float dx = o.Gx - __shfl_down_sync(kFull, o.Gx, 1);
-      const float dy = o.Gy - __shfl_down_sync(kFull, o.Gy, 1);
-      const float dz = o.Gz - __shfl_down_sync(kFull, o.Gz, 1);
-      d1 = {__shfl_sync(kFull, dx, base + 1), __shfl_sync(kFull, dy, base + 1), __shfl_sync(kFull, dz, base + 1)};
-      d2 = {__shfl_sync(kFull, dx, base + 3), __shfl_sync(kFull, dy, base + 3), __shfl_sync(kFull, dz, base + 3)};
-      if (NB == 8) {
-        d3 = {__shfl_sync(kFull, dx, base + 5), __shfl_sync(kFull, dy, base + 5), __shfl_sync(kFull, dz, base + 5)};
-        d4 = {__shfl_sync(kFull, dx, base + 7), __shfl_sync(kFull, dy, base + 7), __shfl_sync(kFull, dz, base + 7)};
-      }
     }
 
     // ------------------------------------------------- central bookkeeping
-    bool emit = false;
-    Vec sr{0.f, 0.f, 0.f}, sk{0.f, 0.f, 0.f}, sa{0.f, 0.f, 0.f}, sb{0.f, 0.f, 0.f};
     if (central && phase != 0) {
-      if (!kTube && emitted && NB > 0) {  // M of the step the neighbours just retraced (Eqs. 9-11)
-        const Vec tp{B.t[0], B.t[1], B.t[2]};
-        const Vec e1p{B.e1[0], B.e1[1], B.e1[2]}, e2p{B.e2[0], B.e2[1], B.e2[2]};
-        Vec c1, c2;
-        if (NB == 2) {  // one-sided: d_j = eps e_j + h^2/6 (G_j - G_0)
-          const float sc = P.h2_6 / B.eps;
-          c1 = {sc * (d1.x - B.g0[0]), sc * (d1.y - B.g0[1]), sc * (d1.z - B.g0[2])};
-          c2 = {sc * (d2.x - B.g0[0]), sc * (d2.y - B.g0[1]), sc * (d2.z - B.g0[2])};
-        } else {        // central difference: d = eps e + h^2/12 (G_+ - G_-)
-          const float sc = P.h2_12 / B.eps;
-          c1 = {sc * d1.x, sc * d1.y, sc * d1.z};
-          c2 = {sc * d2.x, sc * d2.y, sc * d2.z};
-        }
-        float lm = ln_m(c1, c2, e1p, e2p, tp);
-        if (NB == 8) {
-          const float s2 = 0.70710678118654752f, sc = P.h2_12 / B.eps;
-          const Vec g1{s2 * (e1p.x + e2p.x), s2 * (e1p.y + e2p.y), s2 * (e1p.z + e2p.z)};
-          const Vec g2{s2 * (e2p.x - e1p.x), s2 * (e2p.y - e1p.y), s2 * (e2p.z - e1p.z)};
-          const Vec c3{sc * d3.x, sc * d3.y, sc * d3.z}, c4{sc * d4.x, sc * d4.y, sc * d4.z};
-          const float lm2 = ln_m(c3, c4, g1, g2, tp);
-          // M = (M_e + M_g) / 2
-          lm = fmaxf(lm, lm2) + log1p_small(__expf(-fabsf(lm - lm2))) - 0.69314718055994531f;
-        }
-        acc_add<kMixed>(B.lns_hi, B.lns_lo, lm);
-      }
       const float kap = P.emission ? kappa_vac(o.ne1, o.te1, B.kap_c, B.ln_f) : 0.f;
       bool done = false;
       if (phase == 2) {
@@ -520,19 +463,6 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
             done = true;
           }
         }
-        if (!done && P.ckpt && (step % kCkptEvery) == 0) {
-          // state at node `step` for the adjoint's recomputation (bounded by the ray's allocation)
-          const unsigned long long slot = P.ck_off[B.item] + (unsigned long long)(step / kCkptEvery);
-          if (slot < P.ck_off[B.item + 1]) {
-            Ckpt& c = P.ckpt[slot];
-            c.r[0] = px; c.r[1] = py; c.r[2] = pz;
-            c.k[0] = kx; c.k[1] = ky; c.k[2] = kz;
-            c.rl[0] = B.rl[0]; c.rl[1] = B.rl[1]; c.rl[2] = B.rl[2];
-            c.kl[0] = B.kl[0]; c.kl[1] = B.kl[1]; c.kl[2] = B.kl[2];
-            c.tau_hi = B.tau_hi; c.tau_lo = B.tau_lo;
-            c.lns_hi = B.lns_hi; c.lns_lo = B.lns_lo;
-          }
-        }
         if (!done) {
           // complete central step `step` (Eq. 4, RK4 increment form)
           float rlx = B.rl[0], rly = B.rl[1], rlz = B.rl[2];
@@ -540,36 +470,20 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
           const Vec dr{fmaf(h, kx + klx, P.h2_6 * o.Gx), fmaf(h, ky + kly, P.h2_6 * o.Gy),
                        fmaf(h, kz + klz, P.h2_6 * o.Gz)};
           const Vec dk{P.h_6 * o.Ax, P.h_6 * o.Ay, P.h_6 * o.Az};
-          sr = {px, py, pz};
-          sk = {kx, ky, kz};
-          // chord, basis and eps of this step (Eqs. 5, 6, 8)
+          // chord of this step (Eq. 5)
           const float d2n = dot3(dr, dr);
           const float ids = rsqrtf(d2n);
           const Vec tp{dr.x * ids, dr.y * ids, dr.z * ids};
-          if (kTube) {
-            // S_{i+1} = |det[d1, d2, t^i]| (8: mean of the two pairs), ln(S / delta^2)
-            if (B.tube_ok) {
-              const float cx = d1.y * d2.z - d1.z * d2.y, cy = d1.z * d2.x - d1.x * d2.z, cz = d1.x * d2.y - d1.y * d2.x;
-              float S = fabsf(fmaf(tp.x, cx, fmaf(tp.y, cy, tp.z * cz)));
-              if (NB == 8) {
-                const float gx = d3.y * d4.z - d3.z * d4.y, gy = d3.z * d4.x - d3.x * d4.z, gz = d3.x * d4.y - d3.y * d4.x;
-                S = 0.5f * (S + fabsf(fmaf(tp.x, gx, fmaf(tp.y, gy, tp.z * gz))));
-              }
-              B.lns_hi = __logf(S * P.inv_delta2);
-              B.lns_lo = 0.f;
+          // S_{i+1} = |det[d1, d2, t^i]| (8: mean of the two pairs), ln(S / delta^2)
+          if (B.tube_ok) {
+            const float cx = d1.y * d2.z - d1.z * d2.y, cy = d1.z * d2.x - d1.x * d2.z, cz = d1.x * d2.y - d1.y * d2.x;
+            float S = fabsf(fmaf(tp.x, cx, fmaf(tp.y, cy, tp.z * cz)));
+            if (NB == 8) {
+              const float gx = d3.y * d4.z - d3.z * d4.y, gy = d3.z * d4.x - d3.x * d4.z, gz = d3.x * d4.y - d3.y * d4.x;
+              S = 0.5f * (S + fabsf(fmaf(tp.x, gx, fmaf(tp.y, gy, tp.z * gz))));
             }
-          } else if (NB > 0) {
-            Vec e1p, e2p;
-            basis(tp, e1p, e2p);
-            const float eps = (P.eps_fixed > 0.f) ? P.eps_fixed : P.eta * (d2n * ids);
-            B.t[0] = tp.x; B.t[1] = tp.y; B.t[2] = tp.z;
-            B.e1[0] = e1p.x; B.e1[1] = e1p.y; B.e1[2] = e1p.z;
-            B.e2[0] = e2p.x; B.e2[1] = e2p.y; B.e2[2] = e2p.z;
-            B.eps = eps;
-            sa = {eps * e1p.x, eps * e1p.y, eps * e1p.z};
-            sb = {eps * e2p.x, eps * e2p.y, eps * e2p.z};
-            if (NB == 2) { B.g0[0] = o.Gx; B.g0[1] = o.Gy; B.g0[2] = o.Gz; }
-            emit = true;
+            B.lns_hi = __logf(S * P.inv_delta2);
+            B.lns_lo = 0.f;
           }
           Vec rn, kn;
           if (kMixed) {
@@ -605,50 +519,12 @@ __global__ void __launch_bounds__(kThreads, kTube ? kMinBlocksTube : kMinBlocks)
           } else if (!isfinite(rr2 + kn.x + kn.y + kn.z)) {
             B.step = step + 1;
             finish(kNan, rn.x, rn.y, rn.z, B.tb_hi + B.tb_lo);
-            emit = false;
           } else {
             px = rn.x; py = rn.y; pz = rn.z;
             kx = kn.x; ky = kn.y; kz = kn.z;
             B.step = step + 1;
           }
         }
-      }
-      emitted = emit;
-    }
-
-    // ------------------------------------------------- seed broadcast
-    if (!kTube && NB > 0) {
-      const bool e = __shfl_sync(kFull, emit ? 1 : 0, base) != 0;
-      const float bx = __shfl_sync(kFull, sr.x, base), by = __shfl_sync(kFull, sr.y, base),
-                  bz = __shfl_sync(kFull, sr.z, base);
-      const float bkx = __shfl_sync(kFull, sk.x, base), bky = __shfl_sync(kFull, sk.y, base),
-                  bkz = __shfl_sync(kFull, sk.z, base);
-      const float ax = __shfl_sync(kFull, sa.x, base), ay = __shfl_sync(kFull, sa.y, base),
-                  az = __shfl_sync(kFull, sa.z, base);
-      const float cx = __shfl_sync(kFull, sb.x, base), cy = __shfl_sync(kFull, sb.y, base),
-                  cz = __shfl_sync(kFull, sb.z, base);
-      if (used && q > 0) {
-        has_seed = e;
-        // role -> offset: 1 +e1, 2 -e1 (or +e2 with 2 neighbours), 3 +e2, 4 -e2,
-        // 5 +g1, 6 -g1, 7 +g2, 8 -g2 with g1 = (e1+e2)/sqrt2, g2 = (e2-e1)/sqrt2
-        float ox, oy, oz;
-        if (NB == 2) {
-          ox = (q == 1) ? ax : cx; oy = (q == 1) ? ay : cy; oz = (q == 1) ? az : cz;
-        } else if (q <= 4) {
-          const float sgn = (q & 1) ? 1.f : -1.f;
-          ox = sgn * ((q <= 2) ? ax : cx);
-          oy = sgn * ((q <= 2) ? ay : cy);
-          oz = sgn * ((q <= 2) ? az : cz);
-        } else {
-          const float s2 = 0.70710678118654752f;
-          const float sgn = (q & 1) ? 1.f : -1.f;
-          const bool g1 = q <= 6;
-          ox = sgn * s2 * (g1 ? (ax + cx) : (cx - ax));
-          oy = sgn * s2 * (g1 ? (ay + cy) : (cy - ay));
-          oz = sgn * s2 * (g1 ? (az + cz) : (cz - az));
-        }
-        px = bx + ox; py = by + oy; pz = bz + oz;
-        kx = bkx; ky = bky; kz = bkz;
       }
     }
   }

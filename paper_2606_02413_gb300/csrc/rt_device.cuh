@@ -1,5 +1,5 @@
-// Device code of librt: field evaluation, RK4, and the warp-cooperative
-// ray-bundle kernel (Sec. 2.1 Eqs. 4-12, Sec. 3.2 of arXiv 2606.02413).
+// Device code of librt: field evaluation, RK4, transfer helpers and kernel
+// parameters (Sec. 2.1 Eqs. 4-12, Sec. 3.2 of arXiv 2606.02413).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -10,11 +10,7 @@ constexpr float kTwoPiF = 6.28318530717958647692f;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kMaxFreq = 64;
 constexpr int kThreads = 128;
-#ifndef RT_MIN_BLOCKS
-#define RT_MIN_BLOCKS 8
-#endif
-constexpr int kMinBlocks = RT_MIN_BLOCKS;  // __launch_bounds__ occupancy target: 8 x 128 threads per SM
-constexpr int kMinBlocksTube = 6;          // tube bundles: the offset evaluation needs more registers
+constexpr int kMinBlocksTube = 6;  // __launch_bounds__ occupancy target of the tube bundles
 
 // ------------------------------------------------------------------ grid
 // Cells are corner-packed: cell (i, j, k) stores the 8 node values of its
@@ -409,7 +405,7 @@ __device__ __forceinline__ Sample eval_field_off(const GridDev& G, const BasePoi
 
 // ------------------------------------------------------------------- RK4
 // One RK4 step of dr/dtau = k, dk/dtau = kf grad n_e (kf = -C_pe / (2 f^2),
-// i.e. grad(n^2)/2) from (p, k).  Returns G = a1 + a2 + a3 and
+// i.e. grad(n^2)/2) from (p, k): G = a1 + a2 + a3 and
 // A = a1 + 2 a2 + 2 a3 + a4 so that
 //   r' = r + h k + h^2/6 G,   k' = k + h/6 A
 // (the textbook RK4 combination written in increment form), and the stage-1
@@ -419,34 +415,6 @@ struct Rk4Out {
   float ne1, te1;
 };
 
-__device__ __forceinline__ Rk4Out rk4_step(const GridDev& G, float kf, float h, float px, float py,
-                                           float pz, float kx, float ky, float kz, bool want_te) {
-  Rk4Out o;
-  const float hh = 0.5f * h;
-  Sample s = eval_field(G, px, py, pz, want_te);
-  o.ne1 = s.ne;
-  o.te1 = s.te;
-  float ax = kf * s.gx, ay = kf * s.gy, az = kf * s.gz;
-  o.Gx = ax; o.Gy = ay; o.Gz = az;
-  o.Ax = ax; o.Ay = ay; o.Az = az;
-  // stage 2
-  float qx = fmaf(hh, ax, kx), qy = fmaf(hh, ay, ky), qz = fmaf(hh, az, kz);
-  s = eval_field(G, fmaf(hh, kx, px), fmaf(hh, ky, py), fmaf(hh, kz, pz), false);
-  ax = kf * s.gx; ay = kf * s.gy; az = kf * s.gz;
-  o.Gx += ax; o.Gy += ay; o.Gz += az;
-  o.Ax = fmaf(2.f, ax, o.Ax); o.Ay = fmaf(2.f, ay, o.Ay); o.Az = fmaf(2.f, az, o.Az);
-  // stage 3
-  const float q3x = fmaf(hh, ax, kx), q3y = fmaf(hh, ay, ky), q3z = fmaf(hh, az, kz);
-  s = eval_field(G, fmaf(hh, qx, px), fmaf(hh, qy, py), fmaf(hh, qz, pz), false);
-  ax = kf * s.gx; ay = kf * s.gy; az = kf * s.gz;
-  o.Gx += ax; o.Gy += ay; o.Gz += az;
-  o.Ax = fmaf(2.f, ax, o.Ax); o.Ay = fmaf(2.f, ay, o.Ay); o.Az = fmaf(2.f, az, o.Az);
-  // stage 4
-  s = eval_field(G, fmaf(h, q3x, px), fmaf(h, q3y, py), fmaf(h, q3z, pz), false);
-  o.Ax = fmaf(kf, s.gx, o.Ax); o.Ay = fmaf(kf, s.gy, o.Ay); o.Az = fmaf(kf, s.gz, o.Az);
-  return o;
-}
-
 // One RK4 step of a ray of a tube bundle about the base point b, the
 // FP32 node position of the bundle's central ray: the central ray is at
 // b + l (l: the low part of its compensated position, 0 in plain FP32)
@@ -454,7 +422,6 @@ __device__ __forceinline__ Rk4Out rk4_step(const GridDev& G, float kf, float h, 
 // the central lane).  Every stage point is b plus an offset that holds
 // l, the stage's displacement along k and the lane's own offsets, so each
 // evaluation (eval_field_off) resolves it to FP32 precision of the offset.
-// Outputs as rk4_step.
 __device__ __forceinline__ Rk4Out rk4_step_base(const GridDev& G, float kf, float h, const BasePoint& b,
                                                 float lx, float ly, float lz, float kx, float ky, float kz,
                                                 float dpx, float dpy, float dpz, float dkx, float dky,

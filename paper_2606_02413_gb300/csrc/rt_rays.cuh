@@ -15,9 +15,7 @@
 //       retrace of step i for every neighbour, seeded at r^i +- eps e_j with
 //       the central k^i (Eq. 7);
 //   (e) on a clipped last step, closes the path at the crossing point.
-// This is the order of the paper's per-step description; the lane-parallel
-// bundle kernel (rt_bundle.cuh) computes the same quantities with the
-// neighbours one step behind the central lane.
+// This is the order of the paper's per-step description.
 //
 // Why one thread per bundle.  The per-step bookkeeping (basis, ln M,
 // absorption, transfer, termination, compensated updates) is scalar per
@@ -83,7 +81,7 @@ __device__ __forceinline__ Vec rk4_g3_halves(const GridDev& G, float kf, float h
   return sum3(a1, a2, stage3_force(G, kf, hh, p, k, a1));
 }
 
-// One central RK4 step (see rk4_step) with the stage-1 sample including T_e;
+// One central RK4 step (see Rk4Out) with the stage-1 sample including T_e;
 // stages 1 and 2, and then 3 and 4, are independent of each other.  kCurv:
 // also the second derivatives at the first two stage points (cv[0], cv[1]),
 // which the neighbours' retrace needs, and those points' clearance.  The third
