@@ -440,7 +440,8 @@ __device__ __forceinline__ void kappa_partials(float ne, float te, float kap_c, 
 // ------------------------------------------------------------ the kernel
 struct AdjParams {
   GridDev G;
-  float h, h2_6, h_6, h2_12, hrsun, eta, eps_fixed, eps_reach, tbc_K;
+  float h, h2_6, h_6, h2_12, hrsun, eta, eps_fixed, tbc_K;
+  Clear clear;
   int tbc_mode, emission, curv;
   ViewDev view;
   int nf;
@@ -631,8 +632,8 @@ __global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ Adj
       StagePoints sp;
       Rk4Out o;
       if (NB > 0) {
-        const float off_r = radial_reach(P.eps_reach, px, py, pz, kx, ky, kz);
-        o = rk4_central<true>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.eps_reach, &sp);
+        const float off_r = radial_reach(P.clear, px, py, pz, kx, ky, kz);
+        o = rk4_central<true>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.clear.reach, &sp);
       } else {
         o = rk4_central<false>(P.G, kf, h, px, py, pz, kx, ky, kz, 0.f, 0.f, &sp);
       }
@@ -656,7 +657,7 @@ __global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ Adj
         chord_frame(Q, P.eta, P.eps_fixed, dr);
         float c2;
         Q.lm = curvature_ln_m(sp, px, py, pz, Q.t, P.h2_6 * kf, c2);
-        const bool slow = live && !(P.curv && step_clear(sp, Q, dr, P.eps_reach) && c2 <= 1e-8f);
+        const bool slow = live && !(P.curv && step_clear(P.clear, sp, Q, dr) && c2 <= 1e-8f);
         Q.c1 = curvature_dt(sp, px, py, pz, Q.t);
         Q.c2 = {0.f, 0.f, 0.f};
         retrace_shared<NB>(P.G, S.f, slow, kf, h, P.h2_6, P.h2_12, px, py, pz, kx, ky, kz, Q);

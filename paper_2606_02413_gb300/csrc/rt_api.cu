@@ -850,10 +850,17 @@ void fill_common(TraceParams& P, const rt_grid* g, const rt_options* o) {
   P.hrsun = (float)(h * kRsunCm);
   P.eta = (float)o->eta;
   P.eps_fixed = o->eps_mode == 1 ? (float)o->delta : 0.f;
-  // eps = eta |dr| with |dr| ~ h n, n <= 1; a step with a longer chord retraces its neighbours.
-  // 2% for the third stage's own shift (step_clear) and the second order along theta and phi
   P.curv = curvature_form(g, o) ? 1 : 0;
-  P.eps_reach = (float)(1.02 * (o->eps_mode == 1 ? o->delta : o->eta * h));
+  // eps = eta |dr| with |dr| ~ h n, n <= 1; a step with a longer chord retraces its neighbours.
+  // 2% for the third stage's own shift (1% of the reach) and the second order along theta and
+  // phi; a chord that has turned by more than 1% of the reach over eps retraces as well
+  const bool fixed = o->eps_mode == 1;
+  const double reach = 1.02 * (fixed ? o->delta : o->eta * h), near3 = 1e-4 * reach * reach;
+  const double turn = 2.5e-5 * 1.02 * 1.02;  // (1.02 x 1% / 2)^2
+  P.clear.reach = (float)reach;
+  P.clear.pad = fixed ? 0.015f : 0.01f;
+  P.clear.d3 = (float)(fixed ? near3 : std::min(near3, turn * h * h));
+  P.clear.d3_chord = fixed ? (float)turn : std::numeric_limits<float>::max();
   P.tau_stop = (float)o->tau_stop;
   P.max_steps = o->max_steps > 0 ? o->max_steps : (int)std::ceil(40.0 * g->dev.r_max / h);
   P.tbc_mode = o->tbc_mode;
@@ -1258,7 +1265,7 @@ cudaError_t launch_adjoint(rt_ctx* ctx, const rt_grid* g, const TraceParams& P, 
   std::memset(&A, 0, sizeof A);
   A.G = g->dev;
   A.h = P.h; A.h2_6 = P.h2_6; A.h_6 = P.h_6; A.h2_12 = P.h2_12; A.hrsun = P.hrsun;
-  A.eta = P.eta; A.eps_fixed = P.eps_fixed; A.eps_reach = P.eps_reach; A.curv = P.curv; A.tbc_K = P.tbc_K; A.tbc_mode = P.tbc_mode; A.emission = P.emission;
+  A.eta = P.eta; A.eps_fixed = P.eps_fixed; A.clear = P.clear; A.curv = P.curv; A.tbc_K = P.tbc_K; A.tbc_mode = P.tbc_mode; A.emission = P.emission;
   A.view = P.view;
   A.nf = P.nf;
   for (int i = 0; i < P.nf; ++i) A.freq[i] = P.freq[i];

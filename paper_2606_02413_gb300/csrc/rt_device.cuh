@@ -567,12 +567,28 @@ struct Ckpt {
   int step;
 };
 
+// Limits of a step whose neighbours need no retrace (curv).  An eps = eta |dr|
+// shrinks with the chord, which leaves it slack where the chord turns: there 1%
+// of eps for the turn and the rest is enough, and the turn's own limit is one
+// number.  An offset of fixed length needs 1.5%, and the turn held against each
+// chord: near a turning point the force alone sets its direction, and
+// neighbours of rays near the disk centre reached up to 0.3 eps farther than
+// the wave vector says.  Restated in 64 bits over 40 to 300 MHz, rays along and
+// across the radius, steps of 2e-3 to 8e-3 R_sun and both kinds of eps, no
+// neighbour of a step within these limits leaves the reach.
+struct Clear {
+  float reach;     // no neighbour is farther from its ray
+  float pad;       // radially: added to the sine, see radial_reach
+  float d3;        // squared distance of the third stage point from the second, at most
+  float d3_chord;  // and over the squared chord, at most
+};
+
 struct TraceParams {
   GridDev G;
   float h, h2_6, h_6, h2_12, hrsun;  // step and derived constants, hrsun = h R_sun [cm]
   float eta, eps_fixed;              // eps = eta |dr|, or eps_fixed when > 0
   int curv;                          // tube area from the field's second derivatives where a step allows it
-  float eps_reach;                   // curv: no neighbour is farther from its ray (else the step retraces them)
+  Clear clear;
   float tau_stop;                    // <= 0: never
   int max_steps;
   int tbc_mode;

@@ -132,17 +132,15 @@ __device__ __forceinline__ Rk4Out rk4_central(const GridDev& G, float kf, float 
 
 // How far a step's neighbours reach radially: they sit eps off the path
 // across the chord, so eps sin(angle of the ray to the radius), where the wave
-// vector at the node stands for the chord.  0.015 eps more covers the chord's
-// turn away from it and the third stage's shift (0.01 eps each at most, see
-// step_clear), the radius's turn over half a step and the second order
-// eps^2 / 2r; the parts never add up to more (restated in 64 bits over 40 to
-// 300 MHz, rays along and across the radius, 1e-3 to 8e-3 R_sun steps, both
-// kinds of eps).
-__device__ __forceinline__ float radial_reach(float reach, float px, float py, float pz, float kx, float ky, float kz) {
+// vector at the node stands for the chord.  `pad` (of eps, in Clear) covers
+// what that leaves out: the chord's turn and the third stage's shift, which
+// step_clear bounds, the radius's turn over half a step and the second order
+// eps^2 / 2r.
+__device__ __forceinline__ float radial_reach(const Clear& c, float px, float py, float pz, float kx, float ky, float kz) {
   const float pk = fmaf(px, kx, fmaf(py, ky, pz * kz));
   const float pp = fmaf(px, px, fmaf(py, py, pz * pz)), kk = fmaf(kx, kx, fmaf(ky, ky, kz * kz));
   const float c2 = __fdividef(pk * pk, pp * kk);
-  return reach * (__fsqrt_rn(fmaxf(1.f - c2, 0.f)) + 0.015f);
+  return c.reach * (__fsqrt_rn(fmaxf(1.f - c2, 0.f)) + c.pad);
 }
 
 // Trace of the field's Hessian across the direction t at the point (x, y, z):
@@ -215,18 +213,13 @@ __device__ __forceinline__ void chord_frame(Retrace& R, float eta, float eps_fix
 }
 
 // Whether the step's neighbours stay in the cells of the stage points: these
-// are clear of the faces by `reach` (and radial_reach of it), no offset is
-// longer than that, the third stage lies within 1% of it from the second, and
-// the chord has turned from the wave vector (by about h^2/2 |a| / |dr|, twice
-// that distance over the chord) by so little that no neighbour moves by more
-// than 1%.  With eps = eta |dr| and eta <= 1/2 the last follows from the one
-// before; an offset of fixed length needs it near a turning point, where the
-// chord shrinks and the force sets its direction (without it neighbours of
-// rays near the disk centre reached up to 0.3 eps farther than allowed for).
-__device__ __forceinline__ bool step_clear(const StagePoints& sp, const Retrace& R, const Vec& dr, float reach) {
-  const float lim = 1e-4f * reach * reach;
-  return sp.cv[0].clear && sp.cv[1].clear && R.eps <= reach && sp.d3 <= lim &&
-         4.f * sp.d3 * (R.eps * R.eps) <= lim * dot3(dr, dr);
+// are clear of the faces by reach (and radial_reach of it), no offset is
+// longer than that, the third stage lies near the second, and the chord has
+// turned little from the wave vector (by about h^2/2 |a| / |dr|, twice the third
+// stage's distance over the chord): Clear's limits on that distance.
+__device__ __forceinline__ bool step_clear(const Clear& c, const StagePoints& sp, const Retrace& R, const Vec& dr) {
+  // all at once, no short circuit (97x61 x 3 maps with 8 neighbours: 8.0 ms, with && 8.3)
+  return sp.cv[0].clear & sp.cv[1].clear & (sp.d3 <= fminf(c.d3, c.d3_chord * dot3(dr, dr))) & (R.eps <= c.reach);
 }
 
 // c1, c2 and ln M from the raw separations D (NB >= 4: D_j = G_{+j} - G_{-j}
@@ -456,8 +449,8 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
   auto step_once = [&]() {
     // ---------------------------------------------- (a) central RK4 step
     StagePoints sp;
-    const float off_r = kCurv ? radial_reach(P.eps_reach, px, py, pz, kx, ky, kz) : 0.f;
-    const Rk4Out o = rk4_central<kCurv>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.eps_reach, &sp);
+    const float off_r = kCurv ? radial_reach(P.clear, px, py, pz, kx, ky, kz) : 0.f;
+    const Rk4Out o = rk4_central<kCurv>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.clear.reach, &sp);
     const Vec dr = chord(h, P.h2_6, o, kx, ky, kz, klx, kly, klz);
 
     // ---------------------------------------------- (d) ln M of step `step`
@@ -467,7 +460,7 @@ __global__ void __launch_bounds__(kThreads, kRayMinBlocks) trace_rays(const __gr
       chord_frame(R, P.eta, P.eps_fixed, dr);
       float c2;
       R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
-      const bool fast = step_clear(sp, R, dr, P.eps_reach) && c2 <= 1e-6f;
+      const bool fast = step_clear(P.clear, sp, R, dr) && c2 <= 1e-6f;
       retrace_shared<NB>(P.G, slots[threadIdx.x >> 5], active && !fast, kf, h, P.h2_6, P.h2_12, px, py, pz, kx, ky, kz,
                          R);
       lm = R.lm;
@@ -674,8 +667,8 @@ __global__ void __launch_bounds__(kPathThreads)
     float kap_prev = 0.f, te_prev = 0.f, dls = 0.f;
     while (true) {
       StagePoints sp;
-      const float off_r = kCurv ? radial_reach(P.eps_reach, px, py, pz, kx, ky, kz) : 0.f;
-      const Rk4Out o = rk4_central<kCurv>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.eps_reach, &sp);
+      const float off_r = kCurv ? radial_reach(P.clear, px, py, pz, kx, ky, kz) : 0.f;
+      const Rk4Out o = rk4_central<kCurv>(P.G, kf, h, px, py, pz, kx, ky, kz, off_r, P.clear.reach, &sp);
       // the step's end and ln M before the transfer, as in trace_rays: neither
       // waits for its exponentials (256 rays, 4 neighbours: 6.35 -> 6.17 ms)
       const Vec dr = chord(h, P.h2_6, o, kx, ky, kz, klx, kly, klz);
@@ -690,7 +683,7 @@ __global__ void __launch_bounds__(kPathThreads)
           chord_frame(R, P.eta, P.eps_fixed, dr);
           float c2;
           R.lm = curvature_ln_m(sp, px, py, pz, R.t, P.h2_6 * kf, c2);
-          fast = step_clear(sp, R, dr, P.eps_reach) && c2 <= 1e-6f;
+          fast = step_clear(P.clear, sp, R, dr) && c2 <= 1e-6f;
         }
         if (!fast)
           R = retrace_step<(NB > 0 ? NB : 4)>(P.G, kf, h, P.h2_6, P.h2_12, P.eta, P.eps_fixed, px, py, pz, kx, ky,
