@@ -162,10 +162,12 @@ rt_status rt_free_grid(rt_ctx* ctx, rt_grid* grid);
  * thread per bundle in the step-wise forms and with magnification off,
  * adjacent lanes of a warp in tube mode), stepped with RK4, with the tube
  * magnification and the free-free transfer accumulated along the way.
- * With 4 or 8 neighbours and cells wider than their reach, a step whose
- * neighbours stay in the cells of the central ray's stage points takes its
- * magnification from the interpolant's second derivatives there (equal to the
- * retrace's to the third order in eps); the others retrace their neighbours.
+ * With 4 or 8 neighbours, a step whose neighbours stay in the cells of the
+ * central ray's stage points takes its magnification from the interpolant's
+ * second derivatives there (equal to the retrace's to the third order in eps);
+ * the others retrace their neighbours.  All steps do where dtau > 8e-3, where
+ * eps < 50 dtau^2, and where most would: offsets that reach across the cells
+ * or lie within 256 eps of the polar axis over most of the radius.
  * freqs_hz: host, nf entries (1 <= nf <= 64), each > 0.
  * tb_out:   device, [nf][ny][nx] float, caller-owned, fully overwritten.
  * diag:     device, [nf][ny][nx] rt_ray_diag, or NULL.

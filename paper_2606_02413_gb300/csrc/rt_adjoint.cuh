@@ -501,7 +501,9 @@ struct AdjointSlot {
 // the few lanes of a warp that retraced hand their four neighbours to the
 // other lanes, as in the forward.  A step takes its ln M from the second
 // derivatives here where |C| <= 1e-4, so that the first order's derivative
-// errs by less than that.
+// errs by less than that (gradients over steps up to 8e-3 R_sun are as far from
+// 64 bits as with every step retraced); one that the forward took so with a
+// larger |C| is replayed from a retrace, equal to the third order in C.
 //
 // One block holds all the warps of an SM (T / 32 of them at most, see
 // launch_adjoint_rays) and keeps them in the same phase (one
@@ -550,10 +552,10 @@ __global__ void __launch_bounds__(T, 1) adjoint_rays(const __grid_constant__ Adj
   float lkap = 0.f, lte = 0.f;        // partial adjoints of kappa and T_e at the node
   float px = 0.f, py = 0.f, pz = 0.f, kx = 0.f, ky = 0.f, kz = 0.f;  // state of the recomputed step
 
-  // The block's warps meet here (tape and reverse of 128^2 x 8 rays 204 ms on
-  // their own, 165 ms together; 40^2 x 2 rays, one warp a scheduler, 40.3 and
-  // 36.6 ms).  The result passes through a vote, so that the compiler knows it
-  // uniform (the barrier's own: 166 and 37.2 ms).
+  // The block's warps meet here (when measured: tape and reverse of 128^2 x 8
+  // rays 204 ms on their own, 165 ms together; 40^2 x 2 rays, one warp a
+  // scheduler, 40.3 and 36.6 ms).  The result passes through a vote, so that the
+  // compiler knows it uniform (the barrier's own: 166 and 37.2 ms).
   auto any = [&](bool v) { return __any_sync(kFull, __syncthreads_or(v)); };
 
   while (true) {

@@ -1236,9 +1236,11 @@ cudaError_t launch_adjoint_blocks(AdjParams& A, int sm_count, cudaStream_t s) {
 // neighbours).  A step takes a round of either about as long, 1.3 (without
 // neighbours 1.2) times for 16, and a partly filled last round from half of
 // that up, so the rounds that the rays need decide.  Measured (reverse of 8
-// maps, 12 against 16 warps, ms): 51200 rays 55 and 63, 64800 85 and 70,
-// 100352 103 and 124, 131072 137 and 130; without neighbours 26 and 28, 42 and
-// 30, 50 and 55, 68 and 57.
+// maps, 128x90x180 corona at dtau 4e-3, 12 against 16 warps, ms): 28800 rays 27
+// and 30, 51200 34 and 37, 64800 52 and 41, 100352 63 and 72, 131072 84 and 76,
+// 204800 116 and 112 (80000, just past a round of 16, 60 and 51: a miss);
+// without neighbours 12 and 12, 14 and 15, 22 and 16, 26 and 28, 36 and 30, 49
+// and 43.
 template <int NB, bool M>
 cudaError_t launch_adjoint_rays(AdjParams& A, int sm_count, cudaStream_t s) {
   auto rounds = [&](int threads) {

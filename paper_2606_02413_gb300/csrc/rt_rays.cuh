@@ -295,9 +295,10 @@ __device__ __forceinline__ Retrace retrace_step(const GridDev& G, float kf, floa
 // A few second derivatives at two points whose cell and fractions the central
 // ray has anyway cost less than one evaluation.  One GB300, 4 neighbours, global
 // corona 128^2 x 16 frequencies: 660 ms -> 332 ms; 64^2 x 1 on a 64x32x64
-// corona 14.3 -> 7.9 ms; 8 neighbours, 97x61 x 3: 37.5 -> 11.6 ms.  Paths,
-// optical depths and step counts are bit-identical to the retraced form's;
-// ln S differs by 5.6e-8 (rms) on the global corona.
+// corona 14.3 -> 7.9 ms; 8 neighbours, 97x61 x 3: 37.5 -> 11.6 ms (300, 5.5 and
+// 7.7 ms with the steps that came after).  Paths, optical depths and step
+// counts are bit-identical to the retraced form's; ln S differs by 5.6e-8 (rms)
+// on the global corona.
 __device__ __forceinline__ float curvature_ln_m(const StagePoints& sp, float px, float py, float pz, const Vec& t,
                                                 float h2_6kf, float& c2) {
   Vec f1, f2;
