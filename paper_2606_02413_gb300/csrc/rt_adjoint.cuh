@@ -513,9 +513,10 @@ struct AdjointSlot {
 // instruction for it.  One GB300, 128x90x180 corona, 128^2 x 8 frequencies,
 // forward with tape and reverse sweep: 328 ms with 16 force adjoints a step and
 // 128-thread blocks, 223 ms with the second derivatives, 173 ms with one block
-// an SM and the value adjoints in the node's own stage.  Bound by issue and
-// instruction fetch: 210 warp-instructions per ray-step (466 before), of which
-// the shared retraces take about a third.  Where every step is retraced (dtau
+// an SM and the value adjoints in the node's own stage, 150 ms with 12 or 16
+// warps by rounds and each ray's retraces summed into its own accumulator.
+// Bound by latency and issue (54% of the slots): 194 warp-instructions per
+// ray-step (466 before), of which the shared retraces take about a third.  Where every step is retraced (dtau
 // 1e-2, 64x32x64 corona, 320^2 x 2 maps) the reverse sweep takes 60 ms (75 ms
 // with a ray's neighbours one after the other in its own lane).
 template <int NB, bool kMixed, int T>
